@@ -1417,6 +1417,180 @@ k_halo_gather2(const float2* __restrict__ halo, const int* __restrict__ tslot, G
     grid[(size_t)c * geo.G + (size_t)row * geo.g[1] + k1] = sum;
 }
 
+// Run spreading (variant 13, 2D): no tiles and no shared accumulators.  Samples are sorted by the
+// cell of their first tap, rows of a tile one after another, so consecutive samples share most of
+// their footprint.  One warp takes `run` consecutive sorted samples of a group of at most CG
+// coils; lane (j, c, h) owns, of coil c, the grid column congruent to j mod 4 that lies in the
+// current window of four columns, and RPL of its four rows, as sums in registers.  A sample costs
+// two products and 2 RPL FMAs per lane whatever its cell; when the window moves, only the lanes
+// whose column left it add their sums to the grid (red.global.add.v2.f32, 8 coils x up to 4
+// points per instruction, straight to L2) and start the column that entered.
+// A column that a lane finished is held until its aligned block of four columns is, so that the
+// reductions of a dense row go out as whole 32-byte sectors: one column at a time they were
+// 15.9 M sectors and 126 us for 320^2 x 32 coils x 256,000 samples (radial), at the L2's rate of
+// reductions (180 sectors/ns measured); in blocks they are 5.9 M and 98 us, bound by issue (58 % of
+// the slots).  Against the private-tile kernels there is no tile to clear, sum and store, no sample
+// visited once per tile it touches, and no split-tile list: the whole adjoint of that case went from
+// 419 to 177 us, of a spiral 256^2 x 12 coils x 98,304 samples (bf16) from 83.4 to 48.7 us.
+constexpr int RS_WARPS = 8;
+
+template <int CG>
+constexpr size_t run_warp_smem() { return 33 * (2 * sizeof(float4) + (CG + 1) * sizeof(float2) + sizeof(int2)); }
+
+__device__ __forceinline__ void red_add2(float2* p, float2 v) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" :: "l"(p), "f"(v.x), "f"(v.y) : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void lds_vec(const float* p, float* w) {   // N floats, p aligned to their size
+    if (N == 4) { const float4 v = *(const float4*)p; w[0] = v.x; w[1 % N] = v.y; w[2 % N] = v.z; w[3 % N] = v.w; }
+    else if (N == 2) { const float2 v = *(const float2*)p; w[0] = v.x; w[1 % N] = v.y; }
+    else w[0] = *p;
+}
+
+template <int CG, typename UT>
+__device__ __forceinline__ void spread_run_body(const int* __restrict__ k0t, const float* __restrict__ wt,
+                                                const UT* __restrict__ u, const int* __restrict__ perm, const Geom& geo,
+                                                float2* __restrict__ grid, int64_t beg, int64_t end, int c0, int cc,
+                                                unsigned char* sm) {
+    constexpr int RPL = CG / 2, US = CG + 1;              // rows per lane; padded row of staged coil values
+    float4* swy = (float4*)sm;                            // [33] weights of the four rows
+    float4* swx = swy + 33;                               // [33] column weights by column mod 4
+    float2* su = (float2*)(swx + 33);                     // [33][US]
+    int2* sk = (int2*)(su + 33 * US);                     // [33] first tap (row, column)
+    const int lane = threadIdx.x & 31;
+    const int j = lane & 3, c = (lane >> 2) % CG, r0 = (lane >> 2) / CG * RPL;
+    const int g0 = geo.g[0], g1 = geo.g[1];
+    float2* const gc = grid + (size_t)(c0 + c) * geo.G;
+    const bool live = c < cc;
+    // acc: the column 4 (blk + ahead) + j of the current window; pend: the lane's finished column
+    // 4 blk + j, kept until the whole aligned block of four columns is done (when held)
+    float2 acc[RPL], pend[RPL];
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) acc[r] = pend[r] = make_float2(0.f, 0.f);
+    int cy = -1, cx = 0, blk = 0;
+    bool ahead = false, held = false;
+    const auto add = [&](int col, const float2* v) {
+        if (col >= g1) col -= g1;
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) {
+            int row = cy + r0 + r;
+            if (row >= g0) row -= g0;
+            if (live && KP_INB(10, (int64_t)(c0 + c) * geo.G + (int64_t)row * g1 + col, (int64_t)geo.C * geo.G))
+                red_add2(gc + (size_t)row * g1 + col, v[r]);
+        }
+    };
+    const auto zero = [&]() {
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) acc[r] = make_float2(0.f, 0.f);
+    };
+    // adds everything the lanes hold: finished columns, or where a lane has none its current one
+    const auto flush = [&]() {
+        float2 v[RPL];
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) v[r] = held ? pend[r] : acc[r];
+        add(4 * (blk + (ahead && !held ? 1 : 0)) + j, v);
+        if (held) add(4 * (blk + 1) + j, acc);
+    };
+    const auto move = [&](int y, int x) {                 // to the window (y, x), not the current one
+        const bool same = y == cy;
+        const int nb = x >> 2;
+        if (same && nb == blk + 1) {                      // block blk is done
+            float2 v[RPL];
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) v[r] = ahead ? pend[r] : acc[r];
+            if (!ahead || held) add(4 * blk + j, v);
+            if (!ahead) zero();
+            ahead = held = false;
+        } else if (!same || nb != blk) {
+            if (cy >= 0) flush();
+            zero();
+            ahead = held = false;
+            if (j < (x & 3)) ahead = true;                // a new window: nothing was held before it
+        } else if (x < cx) {                              // backwards in the same block (periodic edge)
+            flush();
+            zero();
+            held = false;
+            ahead = j < (x & 3);
+        }
+        if (!ahead && j < (x & 3)) {                      // this lane's column is finished, the next one starts
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) pend[r] = acc[r];
+            zero();
+            ahead = held = true;
+        }
+        cy = y;
+        cx = x;
+        blk = nb;
+    };
+    for (int64_t s0 = beg; s0 < end; s0 += 32) {
+        const int n = (int)(end - s0 < 32 ? end - s0 : 32);
+        __syncwarp();
+        if (lane < n) {
+            const int64_t s = s0 + lane;
+            const int64_t un = perm ? perm[s] : s;
+            const int2 k = make_int2(k0t[s], k0t[geo.M + s]);
+            float w[2 * KW];
+#pragma unroll
+            for (int q = 0; q < 2 * KW; ++q) w[q] = wt[(int64_t)q * geo.M + s];
+            const bool ok = KP_INB(10, un, geo.M);
+            sk[lane] = k;
+            swy[lane] = make_float4(w[0], w[1], w[2], w[3]);
+            // column X carries tap (X - k.y) mod 4: rotate the weights so that index X mod 4 holds it
+            const float a0 = (k.y & 1) ? w[7] : w[4], a1 = (k.y & 1) ? w[4] : w[5];
+            const float a2 = (k.y & 1) ? w[5] : w[6], a3 = (k.y & 1) ? w[6] : w[7];
+            swx[lane] = (k.y & 2) ? make_float4(a2, a3, a0, a1) : make_float4(a0, a1, a2, a3);
+#pragma unroll
+            for (int q = 0; q < CG; ++q)
+                su[lane * US + q] = ok && q < cc ? ldc<UT>(u, (size_t)(c0 + q) * geo.M + un) : make_float2(0.f, 0.f);
+        }
+        __syncwarp();
+        // sample i + 1's staged values are loaded before sample i is used (slot 32 is never used)
+        int2 k = sk[0];
+        float wx = ((const float*)swx)[j];
+        float wy[RPL];
+        lds_vec<RPL>((const float*)swy + r0, wy);
+        float2 uv = su[c];
+#pragma unroll 2
+        for (int i = 0; i < n; ++i) {
+            const int2 kn = k;
+            const float2 v = make_float2(wx * uv.x, wx * uv.y);
+            float wv[RPL];
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) wv[r] = wy[r];
+            k = sk[i + 1];
+            wx = ((const float*)(swx + i + 1))[j];
+            lds_vec<RPL>((const float*)(swy + i + 1) + r0, wy);
+            uv = su[(i + 1) * US + c];
+            if (kn.x != cy || kn.y != cx) move(kn.x, kn.y);   // warp-uniform
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) {
+                acc[r].x = fmaf(wv[r], v.x, acc[r].x);
+                acc[r].y = fmaf(wv[r], v.y, acc[r].y);
+            }
+        }
+    }
+    if (cy >= 0) flush();
+}
+
+// blockIdx.x: RS_WARPS runs of samples; blockIdx.y: group of 8 coils, the last one by the
+// narrowest lane layout that holds its coils.
+template <typename UT>
+__global__ void __launch_bounds__(RS_WARPS * 32)
+k_spread_run(const int* __restrict__ k0t, const float* __restrict__ wt, const UT* __restrict__ u,
+             const int* __restrict__ perm, Geom geo, int run, float2* __restrict__ grid) {
+    __shared__ __align__(16) unsigned char sm[RS_WARPS * run_warp_smem<8>()];
+    const int warp = threadIdx.x >> 5;
+    const int64_t beg = ((int64_t)blockIdx.x * RS_WARPS + warp) * run;
+    const int64_t end = beg + run < geo.M ? beg + run : geo.M;
+    if (beg >= end) return;
+    const int c0 = blockIdx.y * 8, cc = min(8, geo.C - c0);
+    unsigned char* my = sm + warp * run_warp_smem<8>();
+    if (cc > 4) spread_run_body<8, UT>(k0t, wt, u, perm, geo, grid, beg, end, c0, cc, my);
+    else if (cc > 2) spread_run_body<4, UT>(k0t, wt, u, perm, geo, grid, beg, end, c0, cc, my);
+    else spread_run_body<2, UT>(k0t, wt, u, perm, geo, grid, beg, end, c0, cc, my);
+}
+
 // Variant with one shared accumulator per CTA and up to SPA_CH coils per CTA (one coil group
 // for C <= 16): the tap geometry of a sample is staged once for all its coils and the lanes
 // add with shared-memory atomics (a warp's lanes cover distinct (tap, coil) addresses; only
@@ -2065,6 +2239,28 @@ static bool ensure_halo(kp_plan p) {
     return true;
 }
 
+// Samples per warp of the run spreading, in staging rounds of 32: one round, or two once that
+// still leaves every SM 64 warps.  Longer runs save flushes of first and last windows but cost
+// balance: runs in sparse regions add to the grid far more often than runs of the same length in
+// dense ones (320^2 x 32 coils, 256,000 samples: adjoint 177 us with 64-sample runs, 182 with 96,
+// 192 with 160, 203 with 256; below 152 x 64 warps 32 and 64 measured the same).
+static int spread_run_len(const Geom& g) {
+    const int64_t groups = (g.C + 7) / 8;
+    return g.M * groups >= (int64_t)152 * 64 * 64 ? 64 : 32;
+}
+
+// Run spreading, 2D only (variant 13): clears the grid and adds into it.
+template <typename UT>
+static kp_status launch_spread_run(kp_plan p, const UT* u, const int* perm, cudaStream_t st) {
+    const Geom& g = p->geo;
+    if (g.D != 2) { set_error("spreading variant 13 is 2D only"); return KP_EINTERNAL; }
+    KP_TRY_CUDA(cudaMemsetAsync(p->d_grid2, 0, (size_t)g.C * g.G * sizeof(float2), st));
+    const int run = spread_run_len(g);
+    k_spread_run<UT><<<dim3(nblk(g.M, run * RS_WARPS), (g.C + 7) / 8), RS_WARPS * 32, 0, st>>>(p->d_k0, p->d_wt, u, perm, g,
+                                                                                              run, p->d_grid2);
+    return KP_OK;
+}
+
 // Plane-owner spreading, 3D only (variants 8, 9).
 template <int D, typename UT, int CG>
 static kp_status launch_spread_z(kp_plan p, const UT* u, const int* perm, cudaStream_t st) {
@@ -2124,6 +2320,7 @@ static kp_status spread_only(kp_plan p, const void* u, kp_cdtype u_t, const int*
                 case 10: KP_TRY((launch_spread_own<DD, UT, 4>(p, (const UT*)u, perm, st))); break;
                 case 11: KP_TRY((launch_spread_own<DD, UT, 2>(p, (const UT*)u, perm, st))); break;
                 case 12: KP_TRY((launch_spread_own2<UT>(p, (const UT*)u, perm, st))); break;
+                case 13: KP_TRY((launch_spread_run<UT>(p, (const UT*)u, perm, st))); break;
                 default: KP_TRY((launch_spread_priv<DD, UT, 2, 4>(p, (const UT*)u, perm, st))); break;
             }));
     } else if (p->spread_variant == 2) {
@@ -2166,7 +2363,7 @@ kp_status autotune_spread(kp_plan p, cudaStream_t st) {
     if (p->spread_tuned) {
         // a new trajectory may need more slots than the two-phase variants hold: fall back to the
         // private-copy variant, whose lists were not built for a two-phase plan
-        if (p->spread_variant >= 10 && !ensure_halo(p)) {
+        if (p->spread_variant >= 10 && p->spread_variant <= 12 && !ensure_halo(p)) {
             p->spread_variant = 0;
             KP_TRY(build_spread_lists(p, st));
         }
@@ -2182,6 +2379,7 @@ kp_status autotune_spread(kp_plan p, cudaStream_t st) {
         if (v == 2) return wc_ok;
         if (v >= 8 && v <= 11) return g.D == 3 && (v < 10 || own_ok);
         if (v == 12) return g.D == 2 && own_ok;
+        if (v == 13) return g.D == 2;
         return v >= 0 && v <= 7;
     };
     if (!applies(force_v)) force_v = -1;
@@ -2191,7 +2389,7 @@ kp_status autotune_spread(kp_plan p, cudaStream_t st) {
     else chunks = {256, 1024, 4096};
     std::vector<int> variants;
     if (force_v >= 0) variants.push_back(force_v);
-    else for (int v = 0; v <= 12; ++v) if (applies(v)) variants.push_back(v);
+    else for (int v = 0; v <= 13; ++v) if (applies(v)) variants.push_back(v);
     if (chunks.size() == 1 && variants.size() == 1) {
         p->spread_variant = variants[0];
         if (chunks[0] != p->spread_chunk) KP_TRY(build_spread_items(p, chunks[0], st));

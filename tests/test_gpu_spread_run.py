@@ -1,0 +1,38 @@
+"""Run spreading (variant 13): the adjoint against the float64 oracle at the sizes where it can go
+wrong: sample counts around the 32-sample staging rounds and the runs of one warp and one CTA, coil
+groups of 8 and the narrow lane layouts of the last group, grid widths that are and are not
+multiples of the four-column blocks, windows across the periodic edge, many samples in one cell,
+and every storage type of the samples."""
+import numpy as np
+import pytest
+
+from tests.gpu_util import make_plan, need_gpu, random_problem, rel, rounded, to_dev
+from oracle import nufft as onf
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("shape,C,M,kind", [
+    ((16, 16), 1, 1, "c64"), ((16, 18), 2, 31, "c64"), ((21, 34), 3, 32, "bf16"), ((40, 24), 4, 33, "c64"),
+    ((33, 33), 5, 255, "fp16"), ((64, 50), 8, 257, "c64"), ((48, 75), 9, 2049, "c64"), ((24, 24), 12, 5000, "bf16"),
+    ((96, 96), 32, 3001, "c64"), ((12, 12), 6, 160000, "c64"),
+])
+def test_run_spreading_matches_oracle(shape, C, M, kind, monkeypatch):
+    need_gpu()
+    import torch
+    from paper_1902_09657_gb300.api import to_storage
+    monkeypatch.setenv("KPDHG_SPREAD_VARIANT", "13")
+    monkeypatch.setenv("KPDHG_SPREAD_CHUNK", "256")
+    _, maps, traj = random_problem(shape, C, M, seed=M + C, edge=M > 16)
+    if M > 64:
+        traj[:: 3] = traj[0]                       # a third of the samples share one cell
+    rng = np.random.default_rng(M)
+    y = (rng.standard_normal((C, M)) + 1j * rng.standard_normal((C, M))).astype(np.complex64)
+    plan = make_plan(shape, C, M)
+    plan.set_trajectory(to_dev(traj)).set_maps(to_dev(maps))
+    assert plan.spread_config()["variant"] == 13
+    yd = to_storage(torch.from_numpy(y).cuda(), kind)
+    ref = onf.nufft_adjoint(rounded(yd), maps.astype(np.complex128), traj)
+    for _ in range(2):                             # the second call starts from a used grid
+        assert rel(plan.sense_adjoint(yd).cpu().numpy(), ref, "run spreading") < 1e-5
+    plan.close()
