@@ -21,7 +21,7 @@ LIB = os.path.join(HERE, "libkpdhg.so")
 # indices and records an access out of range instead of making it (kp_bounds_report)
 BUILD_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(HERE, "libkpdhg_checked.so")
-SOURCES = ["kp_plan.cu", "kp_nufft.cu", "kp_pdhg.cu", "kp_precond.cu", "kp_wavelet.cu", "kp_unrolled.cu", "kp_noalloc.cu", "kp_batch.cu", "kp_compare.cu", "kp_fft.cu"]
+SOURCES = ["kp_plan.cu", "kp_nufft.cu", "kp_pdhg.cu", "kp_precond.cu", "kp_wavelet.cu", "kp_unrolled.cu", "kp_noalloc.cu", "kp_batch.cu", "kp_compare.cu", "kp_fft.cu", "kp_fft2.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

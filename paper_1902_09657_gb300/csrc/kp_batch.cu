@@ -74,11 +74,15 @@ static kp_status fork_each(kp_batch b, F issue) {
 }
 
 // One PDHG iteration of every case in phase form (issued on the capture stream).
-static kp_status issue_phase_iteration(kp_batch b) {
-    KP_TRY(fork_each(b, [&](int i, cudaStream_t s) { return fft_forward_only(b->plans[i], s); }));
+static kp_status issue_phase_iteration(kp_batch b, const std::vector<int>& regs, const std::vector<float>& lams) {
+    KP_TRY(fork_each(b, [&](int i, cudaStream_t s) { return iteration_forward(b->plans[i], s); }));
     KP_TRY(batch_interp_launch(b->bi, b->cap));
     KP_TRY(batch_spread_launch(b->bi, b->cap));
-    KP_TRY(fork_each(b, [&](int i, cudaStream_t s) { return fft_inverse_only(b->plans[i], s); }));
+    KP_TRY(fork_each(b, [&](int i, cudaStream_t s) {
+        KP_TRY(fft_inverse_only(b->plans[i], s));
+        // the own 2D FFT's last pass is the primal step
+        return b->plans[i]->fft2 ? adjoint_primal(b->plans[i], regs[i], lams[i], s) : KP_OK;
+    }));
     KP_TRY(batch_primal_launch(b->bi, b->cap));
     KP_TRY(batch_wavelet_launch(b->bi, b->cap));
     return batch_pre_launch(b->bi, b->cap);
@@ -95,7 +99,7 @@ static kp_status capture_phase(kp_batch b, const std::vector<int>& regs, const s
     for (const auto& ph : b->bi.inv) nl += ph.nblocks > 0;
     b->phase_launches = nl;
     KP_TRY_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-    const kp_status s = issue_phase_iteration(b);
+    const kp_status s = issue_phase_iteration(b, regs, lams);
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
     if (s != KP_OK) { if (g) cudaGraphDestroy(g); return s; }

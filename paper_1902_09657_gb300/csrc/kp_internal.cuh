@@ -364,6 +364,7 @@ struct Graph {
 };
 
 struct Fft3Plan;                     // kp_fft.cu
+struct Fft2Plan;                     // kp_fft2.cu
 
 }  // namespace kp
 
@@ -443,6 +444,8 @@ struct kp_plan_s {
     cufftHandle fft = 0;
     bool fft_ok = false;
     kp::Fft3Plan* fft3 = nullptr;    // own 3D FFT passes (kp_fft.cu) when the grid sizes allow, else cuFFT
+    kp::Fft2Plan* fft2 = nullptr;    // own 2D passes (kp_fft2.cu) when the grid sizes allow, else cuFFT
+    bool grid2_dirty = false;        // own 2D passes: a spread whose inverse pass (which clears d_grid2) was not issued
     void* d_ystage = nullptr;        // measurements copied in from host memory (kp_pdhg_solve_host)
     size_t ystage_bytes = 0;
     cudaStream_t copy_stream = nullptr;
@@ -528,7 +531,7 @@ kp_status forward_to(kp_plan p, const float2* x, void* out, kp_cdtype out_t, con
 kp_status forward_dual(kp_plan p, const float2* xbar, cudaStream_t st);
 // out = p (A x) in sorted order, divided by sqrt(*n2) when n2 is given (a norm kept on the device)
 kp_status forward_scaled(kp_plan p, const float2* x, float2* out_sorted, const float* ps, cudaStream_t st,
-                         const double* n2 = nullptr);
+                         double* n2 = nullptr);
 // A^H u: u [C][M] (sorted order if perm == nullptr, else user order) -> grid -> x.
 // splits_zeroed: the split tiles' regions of d_grid2 are already zero (the fused primal kernel
 // clears them after its last read of d_grid2, and solve set-up clears them once)
@@ -537,6 +540,7 @@ kp_status adjoint_to_grid(kp_plan p, const void* u, kp_cdtype u_t, const int* pe
 kp_status zero_split_only(kp_plan p, cudaStream_t st);
 kp_status grid_to_image(kp_plan p, float2* x, cudaStream_t st);
 kp_status autotune_spread(kp_plan p, cudaStream_t st);
+void spread_by_rule(kp_plan p);
 kp_status adjoint_primal(kp_plan p, int reg, float lambda, cudaStream_t st);
 kp_status tv_sumabs(kp_plan p, const float2* x, double* out, cudaStream_t st);
 kp_status ensure_tv_dual(kp_plan p);
@@ -585,6 +589,21 @@ kp_status fft3_forward(kp_plan p, const float2* in, float2* out, cudaStream_t st
 // formed by the first pass from x and the maps (no d_grid involved).
 kp_status fft3_forward_image(kp_plan p, const float2* x, cudaStream_t st);
 kp_status fft3_inverse(kp_plan p, float2* io, cudaStream_t st);
+
+// kp_fft2.cu: own 2D FFT with the NUFFT's neighbouring steps fused in (2D plans whose grid lengths
+// factor; KPDHG_FFT=cufft at plan creation keeps cuFFT).  d_grid2 is zero between adjoints.
+kp_status fft2_create(kp_plan p);
+void fft2_destroy(kp_plan p);
+// The forward grid spectrum of image x into d_gridF (coil multiply and apodisation included).  The
+// first kernel also advances *iter (unless null) and shifts nrm[0] = nrm[1], nrm[1] = 0 (unless null).
+kp_status fft2_forward_image(kp_plan p, const float2* x, int* iter, double* nrm, cudaStream_t st);
+// Inverse column pass of d_grid2 into the image rows of d_grid, clearing d_grid2; one of the two
+// row passes below completes the adjoint.
+kp_status fft2_inverse_cols(kp_plan p, cudaStream_t st);
+kp_status fft2_adjoint_image(kp_plan p, float2* x, double* nrm, cudaStream_t st);   // nrm[1] += ||x||^2
+kp_status fft2_adjoint_primal(kp_plan p, int reg, float lambda, cudaStream_t st);
+// Forward FFT of xbar at the start of a PDHG iteration (own 2D passes also advance the counter).
+kp_status iteration_forward(kp_plan p, cudaStream_t st);
 kp_status pre_only(kp_plan p, const float2* x, cudaStream_t st);
 kp_status forward_grid_only(kp_plan p, const float2* x, cudaStream_t st);
 kp_status interp_dual_only(kp_plan p, cudaStream_t st);

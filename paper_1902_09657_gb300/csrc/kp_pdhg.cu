@@ -239,6 +239,9 @@ static kp_status reduce_norm2(kp_plan p, const float2* x, int64_t n, double* out
     return KP_OK;
 }
 
+// Own 2D FFT: squared norms of the power method's last and next vector in d_red.
+constexpr int PW_NRM = 6;
+
 // Power method on A^H P A (Sec. 6: 30 iterations) using the sorted p in d_ps (or none).
 // Start vector in d_z (unnormalised); result L in d_schedd[0].  Each iteration applies
 // A^H P A to w / ||w|| without forming it: the forward pre-step reads w and the interpolation
@@ -248,12 +251,18 @@ static kp_status reduce_norm2(kp_plan p, const float2* x, int64_t n, double* out
 // middle one for all its cases in one graph: begin (norm of the start vector), step (one
 // iteration; the first reads d_z, later ones d_w) and end (L = sqrt of the last norm).
 kp_status power_begin(kp_plan p, cudaStream_t st) {
+    if (p->fft2) return reduce_norm2(p, p->d_z, p->geo.N, p->d_red + PW_NRM + 1, st);
     KP_TRY(zero_split_only(p, st));
     return reduce_norm2(p, p->d_z, p->geo.N, p->d_red, st);
 }
 
 kp_status power_step(kp_plan p, const float* ps_sorted, bool first, cudaStream_t st) {
     const Geom& g = p->geo;
+    if (p->fft2) {             // the norm rides in the adjoint's last pass
+        KP_TRY(forward_scaled(p, first ? p->d_z : p->d_w, p->d_kt, ps_sorted, st, p->d_red + PW_NRM));
+        KP_TRY(adjoint_to_grid(p, p->d_kt, KP_C64, nullptr, st));
+        return fft2_adjoint_image(p, p->d_w, p->d_red + PW_NRM, st);
+    }
     const int n_split = p->spread_variant >= 10 ? 0 : (int)p->n_split;   // 10-12 store every point
     const unsigned nb = (unsigned)std::min<int64_t>(nblk(g.N, 256), 1216);
     KP_TRY(forward_scaled(p, first ? p->d_z : p->d_w, p->d_kt, ps_sorted, st, p->d_red));
@@ -270,7 +279,7 @@ kp_status power_step(kp_plan p, const float* ps_sorted, bool first, cudaStream_t
 }
 
 kp_status power_end(kp_plan p, cudaStream_t st) {
-    k_store_sqrt<<<1, 1, 0, st>>>(p->d_red, p->d_schedd);
+    k_store_sqrt<<<1, 1, 0, st>>>(p->fft2 ? p->d_red + PW_NRM + 1 : p->d_red, p->d_schedd);
     KP_LAUNCH_CHECK();
     p->launches += 1;
     return KP_OK;
@@ -299,8 +308,21 @@ static bool levels_primal(kp_plan p) {
 // FFT -> interpolation + dual update -> spreading + inverse FFT -> fused primal step
 // (adjoint combine, prox, extrapolation, next forward pre-step, counter).
 static kp_status issue_iteration(kp_plan p, int reg, float lambda, cudaStream_t st) {
-    KP_TRY(fft_forward_only(p, st));
+    KP_TRY(iteration_forward(p, st));
     KP_TRY(interp_dual_only(p, st));
+    if (p->fft2) {
+        // own 2D FFT: its first pass formed the pre-step and advanced the counter, its last one
+        // takes the primal step (for l1, z, with the prox after it)
+        KP_TRY(adjoint_to_grid(p, p->d_u, KP_C64, nullptr, st));
+        if (reg != KP_REG_L1_WAVELET) KP_TRY(adjoint_primal(p, reg, lambda, st));
+        else if (cluster_prox_ok(p)) KP_TRY(primal_cluster(p, lambda, st));
+        else {
+            KP_TRY(adjoint_primal(p, reg, lambda, st));
+            KP_TRY(wavelet_prox_levels(p, lambda, st));
+        }
+        mark(p, PH_OTHER, st);
+        return KP_OK;
+    }
     if (reg == KP_REG_TV) {
         // Sec. 4.2: spreading (it clears its split tiles itself), v and x steps, next pre-step
         KP_TRY(adjoint_to_grid(p, p->d_u, KP_C64, nullptr, st, /*splits_zeroed=*/false));
@@ -488,12 +510,13 @@ kp_status solve_setup_b(kp_plan plan, int iters, cudaStream_t st, int reg, const
         if (start) KP_TRY_CUDA(cudaMemcpyAsync(plan->d_v, start->v, (size_t)g.D * g.N * sizeof(float2), cudaMemcpyDeviceToDevice, st));
         else KP_TRY_CUDA(cudaMemsetAsync(plan->d_v, 0, (size_t)g.D * g.N * sizeof(float2), st));   // v_0 = 0
     }
-    k_set_int<<<1, 1, 0, st>>>(plan->d_iter, k0);
+    k_set_int<<<1, 1, 0, st>>>(plan->d_iter, plan->fft2 ? k0 - 1 : k0);   // the own 2D FFT's first pass advances it
     KP_LAUNCH_CHECK();
     plan->launches += 1;
     KP_TRY_CUDA(cudaMemsetAsync(plan->d_bar, 0, 4 * sizeof(unsigned int), st));   // grid-barrier counter
     // forward grid of xbar (the primal step writes the next one each iteration)
-    if (!start) KP_TRY_CUDA(cudaMemsetAsync(plan->d_grid, 0, (size_t)g.C * g.G * sizeof(float2), st));
+    if (plan->fft2) {}      // formed by the first pass of each forward FFT
+    else if (!start) KP_TRY_CUDA(cudaMemsetAsync(plan->d_grid, 0, (size_t)g.C * g.G * sizeof(float2), st));
     else KP_TRY(pre_only(plan, plan->d_xbar, st));
     // split tiles of the spreading grid start at zero (the primal step re-clears them)
     KP_TRY(zero_split_only(plan, st));
@@ -534,6 +557,7 @@ kp_status pdhg_iteration(kp_plan p, int reg, float lambda, cudaStream_t st) { re
 // concurrently): adjoint + primal step kernel, wavelet level kernels (threshold, extrapolation
 // and the next pre-step fused into them) or the pre-step kernel for l2, counter kernel.
 kp_status pdhg_iteration_concurrent(kp_plan p, int reg, float lambda, cudaStream_t st) {
+    if (p->fft2) return issue_iteration(p, reg, lambda, st);
     KP_TRY(fft_forward_only(p, st));
     KP_TRY(interp_dual_only(p, st));
     KP_TRY(adjoint_to_grid(p, p->d_u, KP_C64, nullptr, st));

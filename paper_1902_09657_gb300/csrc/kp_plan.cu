@@ -510,17 +510,20 @@ kp_status plan_create_internal(kp_plan* out, const kp_params* prm, bool unit_map
     KP_A(p->d_schedd, 8);
     KP_A(p->d_iter, 4);
 #undef KP_A
-    int dims[3] = {g.g[0], g.g[1], g.g[2]};
-    cufftResult fr = cufftPlanMany(&p->fft, D, dims, nullptr, 1, (int)G, nullptr, 1, (int)G, CUFFT_C2C, (int)C);
-    if (fr != CUFFT_SUCCESS) {
-        plan_destroy_internal(p);
-        set_error("cufftPlanMany failed: " + std::to_string((int)fr));
-        return fr == CUFFT_ALLOC_FAILED ? KP_ENOMEM : KP_ECUFFT;
-    }
-    p->fft_ok = true;
     {
-        const kp_status fs = fft3_create(p);
+        kp_status fs = fft3_create(p);
+        if (fs == KP_OK) fs = fft2_create(p);
         if (fs != KP_OK) { plan_destroy_internal(p); return fs; }
+    }
+    if (!p->fft3 && !p->fft2) {                     // sizes without own passes
+        int dims[3] = {g.g[0], g.g[1], g.g[2]};
+        cufftResult fr = cufftPlanMany(&p->fft, D, dims, nullptr, 1, (int)G, nullptr, 1, (int)G, CUFFT_C2C, (int)C);
+        if (fr != CUFFT_SUCCESS) {
+            plan_destroy_internal(p);
+            set_error("cufftPlanMany failed: " + std::to_string((int)fr));
+            return fr == CUFFT_ALLOC_FAILED ? KP_ENOMEM : KP_ECUFFT;
+        }
+        p->fft_ok = true;
     }
     if (cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
         plan_destroy_internal(p);
@@ -540,6 +543,7 @@ kp_status plan_destroy_internal(kp_plan p) {
     compare_destroy(p);
     if (p->fft_ok) cufftDestroy(p->fft);
     fft3_destroy(p);
+    fft2_destroy(p);
     void* bufs[] = {p->d_t, p->d_f, p->d_perm, p->d_key, p->d_ccnt, p->d_coff, p->d_scan_part, p->d_scan_poff, p->d_cnt, p->d_off, p->d_ext_off, p->d_ext, p->d_flag,
                     p->d_items, p->d_iitems, p->d_item_off, p->d_slot_off, p->d_nslots, p->d_split, p->d_k0, p->d_wt,
                     p->d_grid2, p->d_gridF, p->d_bar, p->d_tape, p->d_bk,
@@ -743,6 +747,7 @@ kp_status set_trajectory_internal(kp_plan p, const float* traj, float traj_scale
     const Geom& g = p->geo;
     const Tiles& tl = p->tiles;
     const int T = 256;
+    spread_by_rule(p);
     drop_graphs(p);
     p->traj_set = false;
     p->traj_version++;

@@ -523,7 +523,7 @@ kp_status wavelet_prox_levels(kp_plan p, float lambda, cudaStream_t st) {
         if (lev == 0) {
             a.x = p->d_x;
             a.xbar = p->d_xbar;
-            a.fgrid = p->fft3 ? nullptr : p->d_grid;      // the own FFT forms the pre-step itself
+            a.fgrid = p->fft3 || p->fft2 ? nullptr : p->d_grid;      // the own FFT forms the pre-step itself
             a.maps = p->d_maps;
             a.apod = p->d_apod;
             a.geo = g;
@@ -575,7 +575,7 @@ static LevelArgs prox_level_args(kp_plan p, float lambda, int lev, bool fwd, int
         if (lev == 0) {
             a.x = p->d_x;
             a.xbar = p->d_xbar;
-            a.fgrid = p->fft3 ? nullptr : p->d_grid;      // the own FFT forms the pre-step itself
+            a.fgrid = p->fft3 || p->fft2 ? nullptr : p->d_grid;      // the own FFT forms the pre-step itself
             a.maps = p->d_maps;
             a.apod = p->d_apod;
             a.geo = g;
@@ -1167,6 +1167,7 @@ kp_status primal_cluster(kp_plan p, float lambda, cudaStream_t st) {
                                        p->P.wavelet_levels));
     }
     p->launches += 1;
+    if (p->fft2) return KP_OK;      // the next forward FFT forms the pre-step and advances the counter
     mark(p, PH_FWD_PRE, st);
     const int nb_pre = 2 * 152;
     const unsigned nb = (unsigned)(nb_pre + (p->spread_variant >= 10 ? 0 : p->n_split));   // 10-12 store every point
@@ -1198,7 +1199,7 @@ kp_status primal_fused(kp_plan p, int reg, float lambda, cudaStream_t st) {
     a.coef = p->d_w;
     a.ll0 = p->d_wl0;
     a.ll1 = p->d_wl1;
-    a.fgrid = p->fft3 ? nullptr : p->d_grid;            // the own FFT forms the pre-step itself
+    a.fgrid = p->fft3 || p->fft2 ? nullptr : p->d_grid;            // the own FFT forms the pre-step itself
     a.sched = p->d_sched;
     a.iter = p->d_iter;
     a.lambda = lambda;
