@@ -416,7 +416,7 @@ struct kp_plan_s {
     int64_t n_split = 0, split_cap = 0;
     int* d_k0 = nullptr;             // [D][M] wrapped first tap ceil(t) - W/2 per sorted sample
     float* d_wt = nullptr;           // [D * W][M] Kaiser-Bessel weights per sorted sample
-    int chunk = 256;                 // samples per interpolation work item (<= its block size)
+    int chunk = 256;                 // samples per interpolation work item (interp_items_chunk)
     int spread_chunk = 256;          // samples per spreading work item (autotuned, multiple of 256)
     int spread_variant = 0;          // 0/3/4/5: warp-private tiles (coils x warps 4x4, 2x8, 1x8, 2x4);
                                      // 1: shared atomics, 16 coils per CTA; 2: each warp owns 4 coils;
@@ -541,6 +541,7 @@ kp_status zero_split_only(kp_plan p, cudaStream_t st);
 kp_status grid_to_image(kp_plan p, float2* x, cudaStream_t st);
 kp_status autotune_spread(kp_plan p, cudaStream_t st);
 void spread_by_rule(kp_plan p);
+int interp_items_chunk(int D);     // samples per interpolation item
 kp_status adjoint_primal(kp_plan p, int reg, float lambda, cudaStream_t st);
 kp_status tv_sumabs(kp_plan p, const float2* x, double* out, cudaStream_t st);
 kp_status ensure_tv_dual(kp_plan p);

@@ -177,9 +177,9 @@ __global__ void k_fwd_pre(const float2* __restrict__ x, const MT* __restrict__ m
 
 // ---------------------------------------------------------------- forward: interpolation
 // One CTA per (tile chunk, coil group): the grid region the tile's samples read
-// ((ts + W - 1)^D points per coil, periodic) is staged in shared memory by bulk asynchronous
-// copies (cp.async.bulk, one or two per grid row, completing on an mbarrier), then each
-// thread interpolates one sample for the group's coils from shared memory.
+// ((ts + W - 1)^D points per coil, periodic) is staged in shared memory by asynchronous copies
+// completing on an mbarrier, then (2D) each thread interpolates one sample for the group's coils
+// from shared memory; 3D further down.
 constexpr int IP_CH = 4;           // coils per CTA (blockIdx.y selects the group)
 constexpr int IP_THREADS = 256;     // four CTAs per SM (64 registers; 3D: 4 x 46.5 KB staged)
 
@@ -264,20 +264,11 @@ __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)_
 __device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
     asm volatile("mbarrier.init.shared.b64 [%0], %1;" :: "r"(smem_u32(bar)), "r"(count) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_expect_tx(unsigned long long* bar, unsigned bytes) {
-    asm volatile("{ .reg .b64 st; mbarrier.arrive.expect_tx.shared.b64 st, [%0], %1; }"
-                 :: "r"(smem_u32(bar)), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
     unsigned ok;
     asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
                  : "=r"(ok) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return ok != 0;
-}
-// global -> shared bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned)
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 :: "r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 __device__ __forceinline__ bool mbar_test_wait(unsigned long long* bar, unsigned parity) {
     unsigned ok;
@@ -297,14 +288,16 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
 }
 
 // Stages the periodic grid region an interpolation CTA reads ((ts + W - 1)^D points of coils
-// c0 .. c0 + cc - 1, rows of RP points starting at an even x) into sg by bulk asynchronous row
-// copies completing on `bar`; o receives the tile's origin and xo the parity of its first x.
-// The caller waits on bar (bounded).
+// c0 .. c0 + cc - 1, rows of RP points starting at an even x) into sg by 16-byte asynchronous copies
+// completing on `bar`; o receives the tile's origin and xo the parity of its first x.  The caller
+// waits on bar (bounded).  Each thread keeps one 16-byte column of the rows, so a copy costs a table
+// lookup and an add.  (One bulk copy per row issues once per lane, about 25 instructions each: 968
+// copies were two thirds of the instructions of a 3D CTA of 316 samples and 8 coils.)
 template <int D>
 __device__ __forceinline__ void interp_stage(int tile, int c0, int cc, const float2* __restrict__ grid, const Geom& geo,
                                              const Tiles& tl, float2* sg, unsigned long long* bar, int* o, int& xo) {
     using LY = IpL<D>;
-    constexpr int R = LY::R;
+    constexpr int R = LY::R, NCH = LY::RP / 2;               // 16-byte pieces per row
     {
         int r = tile;
 #pragma unroll
@@ -314,76 +307,71 @@ __device__ __forceinline__ void interp_stage(int tile, int c0, int cc, const flo
             o[d] = tc * tl.ts[d];
         }
     }
-    // grid row offsets of the staged region along the slower axes (periodic), computed once
-    __shared__ int rowoff[MAXD][R];
-    if (threadIdx.x < (D - 1) * R) {
-        // axis d < D - 1 without indexing the parameter structs by a thread-dependent d
-        const int d = threadIdx.x / R, l = threadIdx.x % R;
-        const int gd = d == 0 ? geo.g[0] : geo.g[1];
-        const int sd = d == 0 ? tl.sh[0] : tl.sh[1];
-        const int od = d == 0 ? o[0] : o[1 % D];
-        const int stride = D == 3 ? (d == 0 ? geo.g[1] * geo.g[2] : geo.g[2]) : (d == 0 ? geo.g[1] : 1);
-        int pp = od + l;
-        while (pp >= gd) pp -= gd;
-        rowoff[d][l] = tunshift(pp, sd, gd) * stride;
+    // grid offset of every staged row (periodic), computed once
+    __shared__ int rowoff[LY::ROWS];
+    const auto wrapped = [](int p, int sh, int g) {
+        while (p >= g) p -= g;
+        return tunshift(p, sh, g);
+    };
+    for (int q = threadIdx.x; q < LY::ROWS; q += blockDim.x) {
+        if (D == 2) {
+            rowoff[q] = wrapped(o[0] + q, tl.sh[0], geo.g[0]) * geo.g[1];
+        } else {
+            const int z = wrapped(o[0] + q / R, tl.sh[0], geo.g[0]);
+            rowoff[q] = (z * geo.g[1] + wrapped(o[1 % D] + q % R, tl.sh[1], geo.g[1])) * geo.g[2];
+        }
     }
     // first staged x (unshifted), rounded down to even; xo = its parity
     const int gx = geo.g[D - 1];
     const int xs = tunshift(o[D - 1] < gx ? o[D - 1] : o[D - 1] - gx, tl.sh[D - 1], gx);
     xo = xs & 1;
-    const int xlo = xs - xo;
     if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
+        mbar_init(bar, blockDim.x);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    if (threadIdx.x == 0) mbar_arrive_expect_tx(bar, (unsigned)(cc * LY::PER_COIL * sizeof(float2)));
-    for (int j = threadIdx.x; j < cc * LY::ROWS; j += blockDim.x) {
-        const int c = j / LY::ROWS, row = j - c * LY::ROWS;
-        const int off = D == 2 ? rowoff[0][row] : rowoff[0][row / R] + rowoff[1 % (D - 1)][row % R];
-        const float2* src = grid + (size_t)(c0 + c) * geo.G + off;
-        float2* dst = sg + (size_t)j * LY::RP;
-        // the row is periodic: copy up to the grid edge, then continue from x = 0 (pieces
-        // are even in length because the grid extent and the start are even)
-        for (int pos = 0, x = xlo; pos < LY::RP; x = 0) {
-            const int n = min(LY::RP - pos, gx - x);
-            const int64_t o0 = (int64_t)(c0 + c) * geo.G + off + x;
-            // (checked build: a piece out of range copies the grid's first points instead, so the
-            // barrier still receives the bytes it expects)
-            const bool ok = KP_INB(4, o0, (int64_t)geo.C * geo.G) && KP_INB(4, o0 + n - 1, (int64_t)geo.C * geo.G);
-            bulk_g2s(dst + pos, ok ? src + x : grid, (unsigned)(n * sizeof(float2)), bar);
-            pos += n;
+    const int k = threadIdx.x % NCH, r0 = threadIdx.x / NCH, step = blockDim.x / NCH;
+    int x = xs - xo + 2 * k;                                  // the grid extent is even: a piece never crosses its edge
+    while (x >= gx) x -= gx;
+    if (r0 < step) {
+        for (int c = 0; c < cc; ++c) {
+            const float2* src = grid + (size_t)(c0 + c) * geo.G + x;
+            float2* dst = sg + (size_t)c * LY::PER_COIL + 2 * k;
+            for (int row = r0; row < LY::ROWS; row += step) {
+                // (checked build: a piece out of range copies the grid's first points instead)
+                const float2* from = src + rowoff[row];
+                if (!KP_INB(4, (int64_t)(from - grid), (int64_t)geo.C * geo.G - 1)) from = grid;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(smem_u32(dst + row * LY::RP)), "l"(from) : "memory");
+            }
         }
     }
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" :: "r"(smem_u32(bar)) : "memory");
 }
 
 template <int D, int MODE, typename T>
 __device__ __forceinline__ void interp_tile_body(const int4* __restrict__ items, const int* __restrict__ k0t,
                                                  const float* __restrict__ wt, const float2* __restrict__ grid,
-                                                 const Geom& geo, const Tiles& tl, const InterpIO& io, int bx, int by) {
+                                                 const Geom& geo, const Tiles& tl, const InterpIO& io, int bx, int c0) {
     using LY = IpL<D>;
     extern __shared__ __align__(128) float2 sg[];    // [IP_CH][ROWS][RP]
     __shared__ unsigned long long bar;
     const int4 it = items[bx];
     const int tile = it.x, beg = it.y, end = it.z;
-    const int c0 = by * IP_CH;
     const int cc = min(IP_CH, geo.C - c0);
     constexpr int R = LY::R;
     int o[MAXD], xo;
     interp_stage<D>(tile, c0, cc, grid, geo, tl, sg, &bar, o, xo);
     constexpr int rs0 = D == 2 ? LY::RP : R * LY::RP, rs1 = D == 2 ? 1 : LY::RP;
     constexpr int Rtot = LY::PER_COIL;
-    // While the grid region is in flight: this thread's sample (items hold at most blockDim.x
-    // samples), its tap tables and, for the dual step in 2D, its y, p and u.
-    const int s = beg + (int)threadIdx.x;
-    bool act = s < end && KP_INB(5, s, geo.M);
-    float w[D][KW];
-    int lb = xo;
+    // While the grid region is in flight: this thread's (first) sample, its tap tables and, for the
+    // dual step in 2D, its y, p and u.  3D items hold several samples per thread.
     constexpr bool PRE = MODE == 2 && D == 2;     // 3D keeps registers for the 64 taps
+    float w[D][KW];
+    int lb = 0;
     float2 yv[PRE ? IP_CH : 1], uv[PRE ? IP_CH : 1];
     float pv[PRE ? IP_CH : 1];
-    float sigma = 0.f;
-    if (act) {
+    const auto load = [&](int s) {
+        lb = xo;
 #pragma unroll
         for (int d = 0; d < D; ++d) {
             const int p0 = tshift(k0t[(int64_t)d * geo.M + s], tl.sh[d], geo.g[d]);
@@ -391,9 +379,6 @@ __device__ __forceinline__ void interp_tile_body(const int4* __restrict__ items,
 #pragma unroll
             for (int j = 0; j < KW; ++j) w[d][j] = wt[(int64_t)(d * KW + j) * geo.M + s];
         }
-        // the footprint lies in the staged region (the sample's first tap is in this tile)
-        act = KP_INB(4, lb, Rtot) && KP_INB(4, lb + (KW - 1) * (rs0 + (D == 3 ? rs1 : 0) + 1), Rtot);
-        if (MODE == 2) sigma = io.sched[3 * (*io.iter)];
         if (PRE) {
 #pragma unroll
             for (int c = 0; c < IP_CH; ++c) {
@@ -405,13 +390,22 @@ __device__ __forceinline__ void interp_tile_body(const int4* __restrict__ items,
                 }
             }
         }
+    };
+    int s = beg + (int)threadIdx.x;
+    float sigma = 0.f;
+    if (s < end && KP_INB(5, s, geo.M)) {
+        load(s);
+        if (MODE == 2) sigma = io.sched[3 * (*io.iter)];
     }
     if (!mbar_wait_bounded(&bar, 0, io.wait)) {
         if (io.flag) atomicExch(io.flag, 1);
         mbar_wait_bounded(&bar, 0, KP_DRAIN_CYCLES);      // copies still in flight land in this CTA's memory
         return;
     }
-    if (!act) return;
+    for (; s < end && KP_INB(5, s, geo.M); s += IP_THREADS) {
+    if (D == 3 && s >= beg + IP_THREADS) load(s);
+    // the footprint lies in the staged region (the sample's first tap is in this tile)
+    if (!(KP_INB(4, lb, Rtot) && KP_INB(4, lb + (KW - 1) * (rs0 + (D == 3 ? rs1 : 0) + 1), Rtot))) continue;
     // all coils of the group tap by tap: each tap's weight is formed once (no table of 64 weight
     // products held across coils); each coil's sum runs over the taps in the same order
     float2 accs[IP_CH];
@@ -463,13 +457,14 @@ __device__ __forceinline__ void interp_tile_body(const int4* __restrict__ items,
             io.u[os] = make_float2((uo.x + sp * (acc.x - y.x)) * inv, (uo.y + sp * (acc.y - y.y)) * inv);
         }
     }
+    }   // samples
 }
 
 template <int D, int MODE, typename T>
 __global__ void __launch_bounds__(IP_THREADS, 4)
 k_interp_tile(const int4* __restrict__ items, const int* __restrict__ k0t, const float* __restrict__ wt,
-              const float2* __restrict__ grid, Geom geo, Tiles tl, InterpIO io) {
-    interp_tile_body<D, MODE, T>(items, k0t, wt, grid, geo, tl, io, blockIdx.x, blockIdx.y);
+              const float2* __restrict__ grid, Geom geo, Tiles tl, InterpIO io, int c_first) {
+    interp_tile_body<D, MODE, T>(items, k0t, wt, grid, geo, tl, io, blockIdx.x, c_first + blockIdx.y * IP_CH);
 }
 
 // The same over the cases of a batch: block b belongs to the case c with boff[c] <= b <
@@ -480,7 +475,181 @@ k_interp_tile_b(const BInterp* __restrict__ cs, const int* __restrict__ boff, in
     const int c = batch_case(boff, ncase, (int)blockIdx.x);
     const BInterp& a = cs[c];
     const int lb = (int)blockIdx.x - boff[c];
-    interp_tile_body<D, MODE, T>(a.items, a.k0t, a.wt, a.grid, a.geo, a.tl, a.io, lb % a.nx, lb / a.nx);
+    interp_tile_body<D, MODE, T>(a.items, a.k0t, a.wt, a.grid, a.geo, a.tl, a.io, lb % a.nx, lb / a.nx * IP_CH);
+}
+
+// 3D interpolation of 8 coils by runs of samples.  The tile's region is staged as above, and each warp
+// takes 32 sorted samples at a time.  Lane (j, c) holds, of coil c, the column congruent to j mod 4
+// of the current window of four columns: its 4 x 4 (z, y) taps, in registers.  Consecutive samples mostly share a row of cells, so a sample reads from shared
+// memory only the columns that entered the window since the last one (none when it lies in the same
+// cell), plus its z and y weights (one broadcast each), and the x weights and the sum over
+// the four columns are applied to four samples at a time by a transposing shuffle, which leaves
+// lane j with sample j for the epilogue.
+// What bounds it: the shared-memory pipe.  One sample per thread read every tap of every sample from
+// shared memory at 4.4 wavefronts per 32-lane load (unrelated cells in a warp), 413 M wavefronts
+// or 1.31 ms on 192^3 x 8 coils x 6.1 M samples, which is what it took; this form needs about 135 M.
+// @@I
+constexpr int IR_THREADS = 256, IR_S = 32;                  // samples staged per warp
+constexpr int IR_CG = 8;                                    // coils per CTA
+constexpr int IR_CHUNK = 1024;                              // samples per item (a staged region serves them all)
+
+// d = a b + c on two floats at once (one issue slot for a complex value's real and imaginary part)
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{ .reg .b64 x, y, z, w; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mov.b64 z, {%6, %7};\n"
+        "fma.rn.f32x2 w, x, y, z; mov.b64 {%0, %1}, w; }"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
+// Staged samples of one warp: every z and y weight twice (the pair that fma2 multiplies by), x
+// weights by column mod 4, and the window: row offset in the staged region x 32 + first column.
+// Two CTAs of 8 coils just fit an SM (8 x 11.6 KB staged and 21.5 KB of samples each).
+struct IrS {
+    float4 w[IR_S][4];
+    float4 wx[IR_S];
+    int key[IR_S];
+};
+
+static constexpr size_t interp_run_smem() {
+    return (size_t)IR_CG * IpL<3>::PER_COIL * sizeof(float2) + (size_t)(IR_THREADS / 32) * sizeof(IrS);
+}
+
+template <int MODE, typename T>
+__global__ void __launch_bounds__(IR_THREADS, 2)
+k_interp_run3(const int4* __restrict__ items, const int* __restrict__ k0t, const float* __restrict__ wt,
+              const float2* __restrict__ grid, Geom geo, Tiles tl, InterpIO io) {
+    using LY = IpL<3>;
+    constexpr int R = LY::R, RP = LY::RP, CG = IR_CG;
+    extern __shared__ __align__(128) float2 sg[];    // [CG][ROWS][RP], then the warps' staged samples
+    __shared__ unsigned long long bar;
+    const int4 it = items[blockIdx.x];
+    const int c0 = blockIdx.y * CG, cc = min(CG, geo.C - c0);
+    int o[MAXD], xo;
+    interp_stage<3>(it.x, c0, cc, grid, geo, tl, sg, &bar, o, xo);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j = lane & 3, c = lane >> 2;
+    IrS& sm = ((IrS*)(sg + (size_t)CG * LY::PER_COIL))[warp];
+    const float2* const mine = sg + (size_t)min(c, cc - 1) * LY::PER_COIL;
+    const bool live = c < cc;
+    // this lane's coil in the k-space arrays; sample indices stay below 2^26, and below 2^30 in the tap tables
+    const size_t cb = (size_t)(c0 + min(c, cc - 1)) * geo.M;
+    const unsigned M = (unsigned)geo.M;
+    float sigma = 0.f, scale = geo.rsqrtN;
+    if (MODE == 2) sigma = io.sched[3 * (*io.iter)];
+    if (MODE == 1 && io.n2) {
+        const float q = (float)*io.n2;
+        scale *= q > 0.f ? rsqrtf(q) : 0.f;
+    }
+    // a batch's tap tables are loaded one batch ahead (a slot past the end repeats the last sample)
+    unsigned s0 = it.y + warp * IR_S;
+    const unsigned end = it.z;
+    int kk[3];
+    float w[3 * KW];
+    const auto load = [&](unsigned b) {
+        const unsigned s = min(b + lane, end - 1);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) kk[d] = k0t[d * M + s];
+#pragma unroll
+        for (int q = 0; q < 3 * KW; ++q) w[q] = wt[q * M + s];
+    };
+    if (s0 < end) load(s0);
+    if (!mbar_wait_bounded(&bar, 0, io.wait)) {
+        if (io.flag) atomicExch(io.flag, 1);
+        mbar_wait_bounded(&bar, 0, KP_DRAIN_CYCLES);
+        return;
+    }
+    float2 v[KW * KW];                                       // [z][y]
+    int cur = -1, col = -1;                                  // window, this lane's column in it
+    for (; s0 < end; s0 += (IR_THREADS / 32) * IR_S) {
+        const int n = (int)min((unsigned)IR_S, end - s0);
+        __syncwarp();
+        {
+            int l[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                l[d] = tshift(kk[d], tl.sh[d], geo.g[d]) - o[d];
+                if (!KP_INB(4, l[d], tl.ts[d])) l[d] = 0;
+            }
+            const int x = l[2] + xo;
+            sm.key[lane] = (l[0] * R + l[1]) * RP * 32 + x;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sm.w[lane][q] = make_float4(w[2 * q], w[2 * q], w[2 * q + 1], w[2 * q + 1]);
+            // column X carries x tap (X - x) mod 4: rotated so that index X mod 4 holds it
+            const float a0 = (x & 1) ? w[11] : w[8], a1 = (x & 1) ? w[8] : w[9];
+            const float a2 = (x & 1) ? w[9] : w[10], a3 = (x & 1) ? w[10] : w[11];
+            sm.wx[lane] = (x & 2) ? make_float4(a2, a3, a0, a1) : make_float4(a0, a1, a2, a3);
+        }
+        __syncwarp();
+        if (s0 + (IR_THREADS / 32) * IR_S < end) load(s0 + (IR_THREADS / 32) * IR_S);
+        for (int g = 0; g < n; g += 4) {
+            // this lane's sample of the four: what the epilogue reads is in flight meanwhile
+            const unsigned se = s0 + g + j;
+            const bool act = live && g + j < n;
+            float2 yv, uo;
+            float pv = 1.f;
+            int oi = (int)se;
+            if (act) {
+                if (MODE == 0 && io.perm) oi = io.perm[se];
+                if (MODE == 1 && io.ps) pv = (io.ps + cb)[se];
+                if (MODE == 2) { yv = ldc<T>((const T*)io.ys + cb, se); pv = (io.ps + cb)[se]; uo = (io.u + cb)[se]; }
+            }
+            float2 r[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int k = sm.key[g + q];
+                if (k != cur) {                               // warp-uniform
+                    const int x0 = k & 31, x = x0 + ((j - x0) & 3);
+                    if (x != col || (k ^ cur) >> 5) {
+                        col = x;
+                        const float2* a = mine + (k >> 5) + x;
+#pragma unroll
+                        for (int z = 0; z < KW; ++z)
+#pragma unroll
+                            for (int y = 0; y < KW; ++y) v[z * KW + y] = a[(z * R + y) * RP];
+                    }
+                    cur = k;
+                }
+                const float4 z01 = sm.w[g + q][0], z23 = sm.w[g + q][1], y01 = sm.w[g + q][2], y23 = sm.w[g + q][3];
+                const float2 wz[KW] = {{z01.x, z01.y}, {z01.z, z01.w}, {z23.x, z23.y}, {z23.z, z23.w}};
+                const float2 wy[KW] = {{y01.x, y01.y}, {y01.z, y01.w}, {y23.x, y23.y}, {y23.z, y23.w}};
+                float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int z = 0; z < KW; ++z) {
+                    float2 t = make_float2(wy[0].x * v[z * KW].x, wy[0].y * v[z * KW].y);
+#pragma unroll
+                    for (int y = 1; y < KW; ++y) t = fma2(wy[y], v[z * KW + y], t);
+                    acc = fma2(wz[z], t, acc);
+                }
+                const float wx = ((const float*)&sm.wx[g + q])[j];
+                r[q] = make_float2(wx * acc.x, wx * acc.y);
+            }
+            // sum over the four columns; lane j keeps sample g + j
+            const bool b2 = j & 2, b1 = j & 1;
+            float2 a0 = b2 ? r[2] : r[0], a1 = b2 ? r[3] : r[1];
+            const float2 t0 = b2 ? r[0] : r[2], t1 = b2 ? r[1] : r[3];
+            a0.x += __shfl_xor_sync(0xffffffffu, t0.x, 2);
+            a0.y += __shfl_xor_sync(0xffffffffu, t0.y, 2);
+            a1.x += __shfl_xor_sync(0xffffffffu, t1.x, 2);
+            a1.y += __shfl_xor_sync(0xffffffffu, t1.y, 2);
+            float2 sum = b1 ? a1 : a0;
+            const float2 t = b1 ? a0 : a1;
+            sum.x += __shfl_xor_sync(0xffffffffu, t.x, 1);
+            sum.y += __shfl_xor_sync(0xffffffffu, t.y, 1);
+            if (!act || !KP_INB(5, oi, geo.M)) continue;
+            sum.x *= scale;
+            sum.y *= scale;
+            if (MODE == 0) {
+                stc<T>((T*)io.out + cb, oi, sum);
+            } else if (MODE == 1) {
+                (io.outs + cb)[se] = make_float2(sum.x * pv, sum.y * pv);
+            } else {
+                const float sp = sigma * pv;
+                const float inv = 1.f / (1.f + sp);
+                (io.u + cb)[se] = make_float2((uo.x + sp * (sum.x - yv.x)) * inv, (uo.y + sp * (sum.y - yv.y)) * inv);
+            }
+        }
+    }
 }
 
 // ---------------------------------------------------------------- adjoint: spread
@@ -2121,24 +2290,51 @@ kp_status fft_inverse_only(kp_plan p, cudaStream_t st) {
     return grid_fft_inverse(p, st);
 }
 
+// Interpolation launches.  3D coils go in eights to the run kernel; up to four left over (or in all)
+// go to the one-sample-per-thread kernel, whose cost follows the coils, five to seven to the run
+// kernel with idle lanes (128^3 x 2 coils: forward 186 us by sample, 227 us by runs with lanes split
+// over z; 192^3 x 8 coils 2.11 ms by sample, 1.74 ms by runs).
+template <int D, int MODE, typename T>
+static kp_status launch_interp_tile(kp_plan p, const InterpIO& io, int c_first, cudaStream_t st) {
+    static PerDeviceOnce attr;
+    const int left = p->geo.C - c_first;
+    const size_t smem = (size_t)std::min(IP_CH, left) * IpL<D>::PER_COIL * sizeof(float2);
+    if (D == 2 && p->chunk > IP_THREADS) { set_error("interpolation items larger than the block"); return KP_EINTERNAL; }
+    if (attr.first()) KP_TRY_CUDA(cudaFuncSetAttribute(k_interp_tile<D, MODE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
+    k_interp_tile<D, MODE, T><<<dim3((unsigned)p->n_iitems, (left + IP_CH - 1) / IP_CH), IP_THREADS, smem, st>>>(
+        p->d_iitems, p->d_k0, p->d_wt, p->d_gridF, p->geo, p->tiles, io, c_first);
+    return KP_OK;
+}
+
+template <int MODE, typename T>
+static kp_status launch_interp3(kp_plan p, const InterpIO& io, cudaStream_t st) {
+    const int C = p->geo.C, groups = C / IR_CG + (C % IR_CG > IP_CH ? 1 : 0);
+    if (groups > 0) {
+        static PerDeviceOnce attr;
+        if (attr.first())
+            KP_TRY_CUDA(cudaFuncSetAttribute(k_interp_run3<MODE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)interp_run_smem()));
+        k_interp_run3<MODE, T><<<dim3((unsigned)p->n_iitems, groups), IR_THREADS, interp_run_smem(), st>>>(
+            p->d_iitems, p->d_k0, p->d_wt, p->d_gridF, p->geo, p->tiles, io);
+        KP_LAUNCH_CHECK();
+    }
+    if (groups * IR_CG >= C) return KP_OK;
+    if (groups > 0) p->launches += 1;
+    return launch_interp_tile<3, MODE, T>(p, io, groups * IR_CG, st);
+}
+
 template <int MODE>
 static kp_status launch_interp(kp_plan p, kp_cdtype t, const InterpIO& io, cudaStream_t st) {
-    const Geom& g = p->geo;
-    const size_t rt = g.D == 2 ? IpL<2>::PER_COIL : IpL<3>::PER_COIL;
-    const size_t smem = (size_t)IP_CH * rt * sizeof(float2);
-    const dim3 grid((unsigned)p->n_iitems, (g.C + IP_CH - 1) / IP_CH);
-    static PerDeviceOnce attr[2][3][3];
     mark(p, PH_INTERP, st);
     p->launches += 1;
     if (p->n_iitems == 0) return KP_OK;
-    if (p->chunk > IP_THREADS) { set_error("interpolation items larger than the block"); return KP_EINTERNAL; }
-    KP_DISPATCH_D(g.D, DD, KP_DISPATCH_T(t, T,
-        if (attr[DD - 2][MODE][t].first())
-            KP_TRY_CUDA(cudaFuncSetAttribute(k_interp_tile<DD, MODE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-        k_interp_tile<DD, MODE, T><<<grid, IP_THREADS, smem, st>>>(p->d_iitems, p->d_k0, p->d_wt, p->d_gridF, g, p->tiles, io)));
+    KP_DISPATCH_T(t, T,
+        if (p->geo.D == 3) KP_TRY((launch_interp3<MODE, T>(p, io, st)));
+        else KP_TRY((launch_interp_tile<2, MODE, T>(p, io, 0, st))));
     KP_LAUNCH_CHECK();
     return KP_OK;
 }
+
+int interp_items_chunk(int D) { return D == 3 ? IR_CHUNK : SP_CHUNK; }
 
 kp_status forward_to(kp_plan p, const float2* x, void* out, kp_cdtype out_t, const int* perm, cudaStream_t st) {
     KP_TRY(fwd_grid(p, x, st));

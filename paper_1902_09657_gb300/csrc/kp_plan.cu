@@ -384,6 +384,7 @@ kp_status plan_create_internal(kp_plan* out, const kp_params* prm, bool unit_map
     if (!p) { set_error("host allocation failed"); return KP_ENOMEM; }
     p->P = *prm;
     p->unit_maps = unit_maps;
+    p->chunk = interp_items_chunk(D);
     Geom& g = p->geo;
     g.D = D;
     g.C = prm->ncoils;
