@@ -386,7 +386,7 @@ kp_status kp_batch_destroy(kp_batch batch);
  * (diagnostics for load balance). */
 kp_status kp_plan_tile_stats(kp_plan plan, int64_t* ntiles, int64_t* max_tile_samples);
 
-/* The spreading configuration the autotuner chose at the plan's first trajectory: kernel
+/* The spreading configuration chosen at the plan's first trajectory: kernel
  * variant (0: warp-private tile copies, 4 coils x 4 warps per CTA; 1: one shared accumulator
  * with shared-memory atomics, up to 16 coils per CTA; 2: one warp per 4 coils, all coils per
  * CTA; 3, 4, 5: warp-private copies with 2 coils x 8 warps, 1 coil x 8 warps, 2 coils x 4 warps;
@@ -394,7 +394,8 @@ kp_status kp_plan_tile_stats(kp_plan plan, int64_t* ntiles, int64_t* max_tile_sa
  * warp owns one z-plane of a single accumulator, 8 or 4 coils; 10, 11 (3D): two phases, padded
  * tiles of each tile's own samples then a gather over tiles, 8 or 4 coils; 12 (2D): the same two
  * phases with warp-private padded tiles of 4 coils; 13 (2D): runs of sorted samples summed in
- * registers over a moving window and added to the grid, no tiles),
+ * registers over a moving window and added to the grid, no tiles; 14 (3D): the same over padded
+ * tiles; 13 and 14 are the default, and nothing is timed unless a choice is asked for below),
  * samples per work item, number of work items and of split tiles (tiles cut into several items,
  * accumulated with global atomics).  Any pointer may be NULL.  KP_EINVAL before a trajectory
  * is set.  The environment variables KPDHG_SPREAD_VARIANT and KPDHG_SPREAD_CHUNK, read at that

@@ -487,8 +487,8 @@ k_interp_tile_b(const BInterp* __restrict__ cs, const int* __restrict__ boff, in
 // lane j with sample j for the epilogue.
 // What bounds it: the shared-memory pipe.  One sample per thread read every tap of every sample from
 // shared memory at 4.4 wavefronts per 32-lane load (unrelated cells in a warp), 413 M wavefronts
-// or 1.31 ms on 192^3 x 8 coils x 6.1 M samples, which is what it took; this form needs about 135 M.
-// @@I
+// or 1.31 ms on 192^3 x 8 coils x 6.1 M samples, which is what it took; this form takes 0.91 ms, at
+// 76 % of the pipe (30 wavefronts per sample and 8 coils).
 constexpr int IR_THREADS = 256, IR_S = 32;                  // samples staged per warp
 constexpr int IR_CG = 8;                                    // coils per CTA
 constexpr int IR_CHUNK = 1024;                              // samples per item (a staged region serves them all)
@@ -650,6 +650,43 @@ k_interp_run3(const int4* __restrict__ items, const int* __restrict__ k0t, const
             }
         }
     }
+}
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("{ .reg .b64 x, y, w; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5};\n"
+        "add.rn.f32x2 w, x, y; mov.b64 {%0, %1}, w; }"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
+// Reductions into global memory, and small vector loads from shared memory.
+template <int N>
+__device__ __forceinline__ void lds_vec2(const float* p, float* w) {   // 2 N floats, p aligned to min(16, 8 N) bytes
+    if (N == 1) {
+        const float2 v = *(const float2*)p;
+        w[0] = v.x;
+        w[1] = v.y;
+    } else {
+#pragma unroll
+        for (int i = 0; i < N / 2; ++i) {
+            const float4 v = ((const float4*)p)[i];
+            w[4 * i] = v.x; w[(4 * i + 1) % (2 * N)] = v.y; w[(4 * i + 2) % (2 * N)] = v.z; w[(4 * i + 3) % (2 * N)] = v.w;
+        }
+    }
+}
+__device__ __forceinline__ void red_add4(float2* p, float4 v) {       // two complex values, p 16-byte aligned
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" :: "l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void red_add2(float2* p, float2 v) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" :: "l"(p), "f"(v.x), "f"(v.y) : "memory");
+}
+
+template <int N>
+__device__ __forceinline__ void lds_vec(const float* p, float* w) {   // N floats, p aligned to their size
+    if (N == 4) { const float4 v = *(const float4*)p; w[0] = v.x; w[1 % N] = v.y; w[2 % N] = v.z; w[3 % N] = v.w; }
+    else if (N == 2) { const float2 v = *(const float2*)p; w[0] = v.x; w[1 % N] = v.y; }
+    else w[0] = *p;
 }
 
 // ---------------------------------------------------------------- adjoint: spread
@@ -1351,6 +1388,182 @@ k_spread_own(const int* __restrict__ k0t, const float* __restrict__ wt, const UT
     }
 }
 
+// Run spreading in 3D (variant 14).  One CTA of four warps per own-sample item and group of at most
+// CG coils, with one shared accumulator of the padded tile; warp w owns the planes congruent to w
+// mod 4, so each sample has one z tap in every warp and no two warps meet.  Lane (j, c, h) holds,
+// of coil c, the column congruent to j mod 4 of the window of four columns, and RPL of its four
+// rows, as sums in registers: a sample costs its weights, one coil value and RPL multiply-adds, and
+// only the columns that leave the window are added to the accumulator.  At the end the non-zero
+// part of the padded tile is added to the (cleared) grid by 16-byte reductions, halo included, so
+// there are no slots to write and gather (2.6 x the grid's points each way).
+// What bounds it: the shared-memory pipe, by the accumulator's read-modify-writes (64 taps x 8 coils
+// x 16 bytes per run of samples of one cell), at 71 % of its wavefronts, with the issue slots (41
+// instructions per sample and warp) next; 128^3 x 8 coils x 1.7 M samples 0.53 ms.  Measured and not
+// kept: a second pair of warps per plane for the odd rows (16 warps per SM, but the per-sample work
+// repeats: 0.66 ms), and two streams of samples per warp (0.64 ms).  192^3 x 8 coils, whole adjoint:
+// 3.66 -> 3.04 ms.
+constexpr int SC_S = 64, SC_T = 128;           // samples staged at a time, threads
+
+// A staged sample: one pointer reaches all of it, and consecutive records start in different banks.
+struct __align__(16) ScRec {
+    float4 zx[4];              // z x weight products by (plane mod 4, column mod 4)
+    float4 wy[2];              // y weights, each twice (fma2)
+    float2 u[8];               // coil values
+    int at[4];                 // per warp: offset of the window's first point in the accumulator
+};
+
+template <int CG>
+static constexpr size_t spread_cell_smem() {
+    return (size_t)CG * IpL<3>::PER_COIL * sizeof(float2) + (SC_S + 1) * sizeof(ScRec);   // one record that is read ahead only
+}
+
+template <typename UT, int CG>
+__global__ void __launch_bounds__(SC_T)
+k_spread_cell3(const int* __restrict__ k0t, const float* __restrict__ wt, const UT* __restrict__ u,
+               const int* __restrict__ perm, const int4* __restrict__ items, Geom geo, Tiles tl,
+               float2* __restrict__ grid, int c_first) {
+    using LY = IpL<3>;
+    constexpr int R = LY::R, RP = LY::RP, PC = LY::PER_COIL, NCH = RP / 2, NT = SC_T;
+    constexpr int RPL = CG / 2;                              // rows per lane
+    constexpr int ROLES = NT / SC_S;                         // staging threads per sample
+    extern __shared__ __align__(16) float4 smc3[];
+    float2* acc = (float2*)smc3;                             // [CG][R][R][RP]
+    ScRec* rec = (ScRec*)(acc + CG * PC);                    // [SC_S + 1]
+    __shared__ int rowoff[R * R];
+    const int4 it = items[blockIdx.x];
+    const int c0 = c_first + blockIdx.y * CG, cc = min(CG, geo.C - c0);
+    int o[3];
+    {
+        int r = it.x;
+#pragma unroll
+        for (int d = 2; d >= 0; --d) {
+            const int tc = r % tl.nt[d];
+            r /= tl.nt[d];
+            o[d] = tc * tl.ts[d];
+        }
+    }
+    const auto wrapped = [](int p, int sh, int g) {
+        while (p >= g) p -= g;
+        return tunshift(p, sh, g);
+    };
+    for (int q = threadIdx.x; q < R * R; q += NT)
+        rowoff[q] = (wrapped(o[0] + q / R, tl.sh[0], geo.g[0]) * geo.g[1] + wrapped(o[1] + q % R, tl.sh[1], geo.g[1])) * geo.g[2];
+    const int xs = wrapped(o[2], tl.sh[2], geo.g[2]), xo = xs & 1;   // rows start at an even x
+    for (int q = threadIdx.x; q < cc * PC / 2; q += NT) smc3[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int j = lane & 3, c = (lane >> 2) % CG, h = (lane >> 2) / CG;
+    float2* const mine = acc + min(c, cc - 1) * PC + h * RPL * RP;
+    const bool live = c < cc;
+    const unsigned M = (unsigned)geo.M;
+    float2 a[RPL];
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) a[r] = make_float2(0.f, 0.f);
+    // window of this warp's plane, and this lane's first point, in the accumulator.  Row and plane
+    // strides are multiples of 4, so an offset's column is congruent to the offset mod 4.
+    int cur = -1, at = 0;
+    const auto flush = [&]() {
+#pragma unroll
+        for (int r = 0; r < RPL; ++r) {
+            const float2 t = add2(mine[at + r * RP], a[r]);
+            if (live) mine[at + r * RP] = t;
+            a[r] = make_float2(0.f, 0.f);
+        }
+    };
+    const int si = threadIdx.x & (SC_S - 1), role = threadIdx.x / SC_S;   // staging: role 0 the taps, the others y weights and coils
+    for (unsigned s0 = it.y; s0 < (unsigned)it.z; s0 += SC_S) {
+        const int n = (int)min((unsigned)SC_S, (unsigned)it.z - s0);
+        __syncthreads();
+        if (si < n) {
+            const unsigned s = s0 + si;
+            ScRec& q = rec[si];
+            if (role == 0) {
+                int l[3];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    l[d] = tshift(k0t[d * M + s], tl.sh[d], geo.g[d]) - o[d];   // in [0, ts)
+                    if (!KP_INB(7, l[d], tl.ts[d])) l[d] = 0;
+                }
+                const int x = l[2] + xo;
+                float w[KW];
+#pragma unroll
+                for (int e = 0; e < KW; ++e) w[e] = wt[(2 * KW + e) * M + s];
+                // column X holds x tap (X - x) mod 4
+                const float b0 = (x & 1) ? w[3] : w[0], b1 = (x & 1) ? w[0] : w[1];
+                const float b2 = (x & 1) ? w[1] : w[2], b3 = (x & 1) ? w[2] : w[3];
+                const float4 r = (x & 2) ? make_float4(b2, b3, b0, b1) : make_float4(b0, b1, b2, b3);
+#pragma unroll
+                for (int e = 0; e < KW; ++e) {
+                    const float wz = wt[e * M + s];
+                    const int pl = (l[0] + e) & 3;
+                    q.zx[pl] = make_float4(wz * r.x, wz * r.y, wz * r.z, wz * r.w);
+                    q.at[pl] = ((l[0] + e) * R + l[1]) * RP + x;
+                }
+            } else {
+                if (role == 1) {
+                    const float w0 = wt[KW * M + s], w1 = wt[(KW + 1) * M + s], w2 = wt[(KW + 2) * M + s], w3 = wt[(KW + 3) * M + s];
+                    q.wy[0] = make_float4(w0, w0, w1, w1);
+                    q.wy[1] = make_float4(w2, w2, w3, w3);
+                }
+                const int64_t un = perm ? perm[s] : s;
+                const bool ok = KP_INB(6, un, geo.M);
+#pragma unroll
+                for (int e = role - 1; e < CG; e += ROLES - 1)
+                    q.u[e] = ok && e < cc ? ldc<UT>(u, (size_t)(c0 + e) * geo.M + un) : make_float2(0.f, 0.f);
+            }
+        }
+        __syncthreads();
+        // sample i + 1's record is loaded before sample i is used
+        const ScRec* q = rec;
+        int k = q->at[warp];
+        float zx = ((const float*)&q->zx[warp])[j];
+        float wy[2 * RPL];
+        lds_vec2<RPL>((const float*)q->wy + 2 * h * RPL, wy);
+        float2 uv = q->u[c];
+#pragma unroll 2
+        for (int i = 0; i < n; ++i) {
+            const int kn = k;
+            const float2 v = make_float2(zx * uv.x, zx * uv.y);
+            float wv[2 * RPL];
+#pragma unroll
+            for (int r = 0; r < 2 * RPL; ++r) wv[r] = wy[r];
+            ++q;
+            k = q->at[warp];
+            zx = ((const float*)&q->zx[warp])[j];
+            lds_vec2<RPL>((const float*)q->wy + 2 * h * RPL, wy);
+            uv = q->u[c];
+            if (kn != cur) {                                 // warp-uniform
+                const int to = kn + ((j - kn) & 3);
+                if (to != at) {
+                    flush();                                 // (the first time zeros, to a point of the tile)
+                    at = to;
+                }
+                cur = kn;
+                if (CG < 8) __syncwarp();                    // another lane may hold the row next
+            }
+#pragma unroll
+            for (int r = 0; r < RPL; ++r) a[r] = fma2(make_float2(wv[2 * r], wv[2 * r + 1]), v, a[r]);
+        }
+    }
+    flush();
+    __syncthreads();
+    // padded tile -> grid: each thread keeps one 16-byte column of the rows
+    const int kc = threadIdx.x % NCH, q0 = threadIdx.x / NCH;
+    constexpr int step = NT / NCH;
+    int x = xs - xo + 2 * kc;
+    while (x >= geo.g[2]) x -= geo.g[2];
+    if (q0 >= step) return;
+    for (int q = 0; q < cc; ++q) {
+        float2* dst = grid + (size_t)(c0 + q) * geo.G + x;
+        const float4* src = (const float4*)(acc + q * PC) + kc;
+        for (int row = q0; row < R * R; row += step) {
+            const float4 v = src[row * NCH];
+            if ((v.x != 0.f || v.y != 0.f || v.z != 0.f || v.w != 0.f) &&
+                KP_INB(9, (int64_t)(c0 + q) * geo.G + rowoff[row] + x, (int64_t)geo.C * geo.G - 1))
+                red_add4(dst + rowoff[row], v);
+        }
+    }
+}
+
 // Phase B: one CTA per tile (empty tiles included, so every grid point is stored once).  The
 // tile's value is the sum of its own slots' 8^3 cores and of the halos that its 7 lower
 // neighbours (periodic) spill into it: the neighbour across axis set m covers the sub-box with
@@ -1605,17 +1818,6 @@ constexpr int RS_WARPS = 8;
 
 template <int CG>
 constexpr size_t run_warp_smem() { return 33 * (2 * sizeof(float4) + (CG + 1) * sizeof(float2) + sizeof(int2)); }
-
-__device__ __forceinline__ void red_add2(float2* p, float2 v) {
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" :: "l"(p), "f"(v.x), "f"(v.y) : "memory");
-}
-
-template <int N>
-__device__ __forceinline__ void lds_vec(const float* p, float* w) {   // N floats, p aligned to their size
-    if (N == 4) { const float4 v = *(const float4*)p; w[0] = v.x; w[1 % N] = v.y; w[2 % N] = v.z; w[3 % N] = v.w; }
-    else if (N == 2) { const float2 v = *(const float2*)p; w[0] = v.x; w[1 % N] = v.y; }
-    else w[0] = *p;
-}
 
 template <int CG, typename UT>
 __device__ __forceinline__ void spread_run_body(const int* __restrict__ k0t, const float* __restrict__ wt,
@@ -2479,6 +2681,36 @@ static kp_status launch_spread_run(kp_plan p, const UT* u, const int* perm, cuda
     return KP_OK;
 }
 
+// Run spreading, 3D only (variant 14): clears the grid and adds into it; coils in eights, the rest by
+// the narrowest lane layout that holds them.
+template <int D, typename UT, int CG>
+static kp_status launch_spread_cell(kp_plan p, const UT* u, const int* perm, int c_first, int groups, cudaStream_t st) {
+    static PerDeviceOnce attr;
+    const size_t sm = spread_cell_smem<CG>();
+    if (attr.first()) KP_TRY_CUDA(cudaFuncSetAttribute(k_spread_cell3<UT, CG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    if (p->n_oitems > 0 && groups > 0)
+        k_spread_cell3<UT, CG><<<dim3((unsigned)p->n_oitems, groups), SC_T, sm, st>>>(p->d_k0, p->d_wt, u, perm, p->d_oitems,
+                                                                                     p->geo, p->tiles, p->d_grid2, c_first);
+    KP_LAUNCH_CHECK();
+    return KP_OK;
+}
+
+template <int D, typename UT>
+static kp_status launch_spread_run3(kp_plan p, const UT* u, const int* perm, cudaStream_t st) {
+    const Geom& g = p->geo;
+    if (D != 3 || p->tiles.ts[0] > 8 || p->tiles.ts[1] > 8 || p->tiles.ts[2] > 8) {
+        set_error("spreading variant 14 needs a 3D plan with tiles of at most 8");
+        return KP_EINTERNAL;
+    }
+    KP_TRY_CUDA(cudaMemsetAsync(p->d_grid2, 0, (size_t)g.C * g.G * sizeof(float2), st));
+    const int r = g.C % 8, full = g.C / 8 + (r > 4 ? 1 : 0);
+    KP_TRY((launch_spread_cell<D, UT, 8>(p, u, perm, 0, full, st)));
+    if (r == 0 || r > 4) return KP_OK;
+    if (full > 0) p->launches += 1;
+    if (r > 2) return launch_spread_cell<D, UT, 4>(p, u, perm, full * 8, 1, st);
+    return launch_spread_cell<D, UT, 2>(p, u, perm, full * 8, 1, st);
+}
+
 // Plane-owner spreading, 3D only (variants 8, 9).
 template <int D, typename UT, int CG>
 static kp_status launch_spread_z(kp_plan p, const UT* u, const int* perm, cudaStream_t st) {
@@ -2546,6 +2778,7 @@ static kp_status spread_only(kp_plan p, const void* u, kp_cdtype u_t, const int*
                 case 11: KP_TRY((launch_spread_own<DD, UT, 2>(p, (const UT*)u, perm, st))); break;
                 case 12: KP_TRY((launch_spread_own2<UT>(p, (const UT*)u, perm, st))); break;
                 case 13: KP_TRY((launch_spread_run<UT>(p, (const UT*)u, perm, st))); break;
+                case 14: KP_TRY((launch_spread_run3<DD, UT>(p, (const UT*)u, perm, st))); break;
                 default: KP_TRY((launch_spread_priv<DD, UT, 2, 4>(p, (const UT*)u, perm, st))); break;
             }));
     } else if (p->spread_variant == 2) {
@@ -2577,13 +2810,15 @@ kp_status adjoint_to_grid(kp_plan p, const void* u, kp_cdtype u_t, const int* pe
     return grid_fft_inverse(p, st);
 }
 
-// 2D plans spread by runs: on every case measured (adjoints of 76^2 x 3 to 320^2 x 32 coils) it was
-// the fastest variant, the closest 128^2 x 4 coils, 26.8 against 28.2 us while it still needed a
-// separate clear.  So nothing is timed, and the tile lists of the other variants are not built,
-// unless a variant or an item size is asked for by the environment.
+// Plans spread by runs: on every case measured it was the fastest variant, in 2D (adjoints of 76^2 x
+// 3 to 320^2 x 32 coils; the closest 128^2 x 4 coils, 26.8 against 28.2 us while it still needed a
+// separate clear) and in 3D (48^3 x 6 coils 61 against 100 us, 64^3 x 12 321 against 516, 128^3 x 1 234
+// against 337, 150 x 132 x 116 x 5 1.79 against 1.98 ms, 192^3 x 8 3.04 against 3.66 ms).  So nothing is
+// timed, and the tile lists and slots of the other variants are not built, unless a variant or an
+// item size is asked for by the environment.
 void spread_by_rule(kp_plan p) {
-    if (p->spread_tuned || p->geo.D != 2 || getenv("KPDHG_SPREAD_VARIANT") || getenv("KPDHG_SPREAD_CHUNK")) return;
-    p->spread_variant = 13;
+    if (p->spread_tuned || getenv("KPDHG_SPREAD_VARIANT") || getenv("KPDHG_SPREAD_CHUNK")) return;
+    p->spread_variant = p->geo.D == 2 ? 13 : 14;
     p->spread_tuned = true;
 }
 
@@ -2615,6 +2850,7 @@ kp_status autotune_spread(kp_plan p, cudaStream_t st) {
         if (v >= 8 && v <= 11) return g.D == 3 && (v < 10 || own_ok);
         if (v == 12) return g.D == 2 && own_ok;
         if (v == 13) return g.D == 2;
+        if (v == 14) return g.D == 3;
         return v >= 0 && v <= 7;
     };
     if (!applies(force_v)) force_v = -1;
@@ -2624,7 +2860,7 @@ kp_status autotune_spread(kp_plan p, cudaStream_t st) {
     else chunks = {256, 1024, 4096};
     std::vector<int> variants;
     if (force_v >= 0) variants.push_back(force_v);
-    else for (int v = 0; v <= 13; ++v) if (applies(v)) variants.push_back(v);
+    else for (int v = 0; v <= 14; ++v) if (applies(v)) variants.push_back(v);
     if (chunks.size() == 1 && variants.size() == 1) {
         p->spread_variant = variants[0];
         if (chunks[0] != p->spread_chunk) KP_TRY(build_spread_items(p, chunks[0], st));

@@ -1,4 +1,4 @@
-"""Run spreading (variant 13): the adjoint against the float64 oracle at the sizes where it can go
+"""Run spreading (variants 13 and 14): the adjoint against the float64 oracle at the sizes where it can go
 wrong: sample counts around the 32-sample staging rounds and the runs of one warp and one CTA, coil
 groups of 8 and the narrow lane layouts of the last group, grid widths that are and are not
 multiples of the four-column blocks, windows across the periodic edge, many samples in one cell,
@@ -35,4 +35,28 @@ def test_run_spreading_matches_oracle(shape, C, M, kind, monkeypatch):
     ref = onf.nufft_adjoint(rounded(yd), maps.astype(np.complex128), traj)
     for _ in range(2):                             # the second call starts from a used grid
         assert rel(plan.sense_adjoint(yd).cpu().numpy(), ref, "run spreading") < 1e-5
+    plan.close()
+
+
+@pytest.mark.parametrize("shape,C,M,kind", [
+    ((16, 16, 16), 8, 1, "c64"), ((20, 16, 20), 5, 63, "bf16"), ((16, 20, 20), 1, 64, "c64"), ((24, 16, 18), 2, 65, "fp16"),
+    ((20, 20, 20), 4, 129, "c64"), ((12, 24, 16), 9, 2051, "c64"), ((16, 16, 16), 11, 700, "bf16"), ((30, 24, 26), 16, 5003, "c64"),
+    ((8, 9, 10), 6, 3000, "c64"), ((16, 16, 16), 8, 40001, "c64"),
+])
+def test_run_spreading_3d_matches_oracle(shape, C, M, kind):
+    need_gpu()
+    import torch
+    from paper_1902_09657_gb300.api import to_storage
+    _, maps, traj = random_problem(shape, C, M, seed=M + C, edge=M > 16)
+    if M > 64:
+        traj[::3] = traj[0]
+    rng = np.random.default_rng(M)
+    y = (rng.standard_normal((C, M)) + 1j * rng.standard_normal((C, M))).astype(np.complex64)
+    plan = make_plan(shape, C, M)
+    plan.set_trajectory(to_dev(traj)).set_maps(to_dev(maps))
+    assert plan.spread_config()["variant"] == 14
+    yd = to_storage(torch.from_numpy(y).cuda(), kind)
+    ref = onf.nufft_adjoint(rounded(yd), maps.astype(np.complex128), traj)
+    for _ in range(2):
+        assert rel(plan.sense_adjoint(yd).cpu().numpy(), ref, "run spreading 3D") < 1e-5
     plan.close()
