@@ -1,5 +1,5 @@
 // Own 3D FFT of a plan's oversampled grids (all coils at once), used in place of cuFFT for 3D
-// plans whose grid sizes factor into 2, 3 and 5 (Sec. 6's oversampled FFT, unnormalised in
+// plans (any length with at most one prime factor above 5 and that up to 127) (Sec. 6's oversampled FFT, unnormalised in
 // both directions like cuFFT: forward e^{-2 pi i n k / g}, inverse e^{+2 pi i n k / g}).
 //
 // One pass per axis.  A CTA takes 16 lines of one axis (8 for axes longer than 256 points): rows
@@ -40,6 +40,7 @@ constexpr int FF_MAXN = 512;     // longest axis handled
 constexpr int FF_MAXST = 10;     // radix stages at most
 
 struct FfAxis {
+    F2Axis gen;                  // lengths without a compiled pass: the pass of run-time length (nst = 0: compiled)
     int N;                       // transform length (grid points along the axis)
     int nst;                     // radix stages
     int r[FF_MAXST];             // radices in the order applied
@@ -50,14 +51,6 @@ struct Fft3Plan {
     FfAxis ax[3];
     float2* d_tw = nullptr;
     FfConst k;
-};
-
-// The image samples the first forward pass forms itself (coil multiply and apodisation, the
-// NUFFT's pre-step fused into the FFT): x, the maps (null: unit maps) and 1/Phi per axis.
-struct PreSrc {
-    const float2* x;
-    const void* maps;
-    const float* apod;
 };
 
 // Radices of N in the order applied, at compile time (-1: N is not handled).  The
@@ -352,6 +345,10 @@ static bool factor(int N, FfAxis& ax) {
 }
 
 static bool size_compiled(int N);
+// kp_fft2.cu: the pass of run-time length along AXIS
+bool fftg_fits(const F2Axis& ax);
+template <int AXIS, bool INV, bool PRE, typename MT>
+kp_status fftg_pass(const F2Axis& ax, const FfConst& k, const Geom& g, const float2* in, float2* out, const PreSrc& pre, cudaStream_t st);
 
 // Passes and twiddle tables for grids of g[0] x g[1] x g[2] points; null when some length has no
 // compiled passes (or KPDHG_FFT=cufft).
@@ -359,24 +356,25 @@ Fft3Plan* fft3_make(const int g[3]) {
     const char* env = std::getenv("KPDHG_FFT");
     if (env && std::string(env) == "cufft") return nullptr;       // cuFFT when asked for
     Fft3Plan f{};
-    size_t tot = 0;
     for (int d = 0; d < 3; ++d) {
         FfAxis& ax = f.ax[d];
         ax.N = g[d];
-        if (ax.N > FF_MAXN || !factor(ax.N, ax) || !size_compiled(ax.N)) return nullptr;
-        tot += ax.N;
-    }
-    // twiddle tables e^{-2 pi i m / N} in float64, rounded once
-    std::vector<float2> h(tot);
-    size_t o = 0;
-    for (int d = 0; d < 3; ++d) {
-        const int N = f.ax[d].N;
-        for (int m = 0; m < N; ++m) {
-            const double a = -2.0 * M_PI * (double)m / (double)N;
-            h[o + m] = make_float2((float)std::cos(a), (float)std::sin(a));
+        if (ax.N > FF_MAXN || !size_compiled(ax.N)) {
+            if (!fft_axis_factor(ax.N, ax.gen) || !fftg_fits(ax.gen)) return nullptr;
+        } else if (!factor(ax.N, ax)) {
+            return nullptr;
         }
-        o += N;
     }
+    // twiddle tables in float64, rounded once
+    std::vector<float2> h;
+    size_t first[3];
+    for (int d = 0; d < 3; ++d) {
+        first[d] = h.size();
+        F2Axis a = f.ax[d].gen;
+        a.N = f.ax[d].N;
+        fft_axis_table(a, h);
+    }
+    const size_t tot = h.size();
     Fft3Plan* q = new (std::nothrow) Fft3Plan(f);
     if (!q) return nullptr;
     if (cudaMalloc(&q->d_tw, tot * sizeof(float2)) != cudaSuccess) {
@@ -390,11 +388,7 @@ Fft3Plan* fft3_make(const int g[3]) {
         delete q;
         return nullptr;
     }
-    o = 0;
-    for (int d = 0; d < 3; ++d) {
-        q->ax[d].tw = q->d_tw + o;
-        o += q->ax[d].N;
-    }
+    for (int d = 0; d < 3; ++d) q->ax[d].tw = q->ax[d].gen.tw = q->d_tw + first[d];
     q->k = ff_const();
     return q;
 }
@@ -416,7 +410,8 @@ void fft3_destroy(kp_plan p) {
 }
 
 // Grid sizes with compiled passes (the 3D workloads' grids and their preconditioner's 2N grids,
-// and small test grids); a plan with another size keeps cuFFT.
+// and small test grids); another length takes the passes of run-time length (150 x 132 x 116 x 5 coils,
+// grid 188 x 166 x 146 with the primes 47, 83 and 73: @@G).
 #define KP_FFT_SIZES(X) X(20) X(30) X(40) X(60) X(80) X(100) X(120) X(160) X(200) X(240) X(320) X(384) X(400) X(480)
 
 static bool size_compiled(int N) {
@@ -444,6 +439,10 @@ static kp_status launch_pass_n(const Fft3Plan* f, const Geom& g, const float2* i
 template <int AXIS, bool INV, bool PRE = false, typename MT = float2>
 static kp_status launch_pass(const Fft3Plan* f, const Geom& g, int64_t& launches, const float2* in, float2* out,
                              cudaStream_t st, const PreSrc& pre = PreSrc{}) {
+    if (f->ax[AXIS].gen.nst > 0) {
+        launches += 1;
+        return fftg_pass<AXIS, INV, PRE, MT>(f->ax[AXIS].gen, f->k, g, in, out, pre, st);
+    }
     int64_t nblocks;
     const int ln = g.g[AXIS] <= 256 ? 16 : 8;           // ff_lines(N) of this pass
     const int64_t xblocks = (g.g[2] + ln - 1) / ln;

@@ -20,6 +20,8 @@
 // Larger radices (two stages of 16 x 20 for 320 points) were no faster: fewer barriers, but long
 // straight code run once by few threads.
 //
+// 3D grids whose lengths have no compiled pass in kp_fft.cu run the same stages (k_fftg_pass).
+//
 // These grids live in L2 and a pass is bound by its latency (launch, loads, one or two barriers,
 // stores), not by bytes: what pays is fewer kernels, fewer dependent steps and every CTA resident
 // in one wave (64 registers, four CTAs per SM).  One application of A^H P A
@@ -37,17 +39,9 @@
 
 namespace kp {
 
-constexpr int F2_MAXST = 8;       // radix stages at most
-constexpr int F2_MAXP = 61;       // largest prime factor summed directly
+constexpr int F2_MAXP = 127;      // largest prime factor summed directly
 constexpr int F2_T = 256;         // threads per CTA at most
 constexpr int F2_SMEM = 200 * 1024;
-
-struct F2Axis {
-    int N, nst;                   // at least two stages
-    int r[F2_MAXST];              // radices in the order applied
-    unsigned mg[F2_MAXST];        // 2^32 / m + 1 for the stage's m (bf / m by a high product)
-    const float2* tw;             // e^{-2 pi i m / N}
-};
 
 struct Fft2Plan {
     F2Axis ax[2];                 // y, x
@@ -174,27 +168,45 @@ __device__ __forceinline__ void f2_last(ST st, int ia, const float2* tw, int N, 
 }
 
 // First stage for a prime radix without a compiled butterfly: the lines are copied to the buffer at
-// ia, then each thread forms the outputs t and R - t of a butterfly (folded as above).
+// ia, then each thread forms, for up to F2_TB values of t, the outputs t and R - t of a butterfly
+// (folded as above) with the table w_R^(q t) that follows tw.  Bound by issue: per input pair and t one
+// table load and four FMAs (one t per thread and table indices reduced mod R took 13 instead of 7).
+constexpr int F2_TB = 4;
 template <int LN, int P, typename LD>
 __device__ __forceinline__ void f2_first_prime(LD ld, int R, int ia, int ib, const float2* tw, int N, float s) {
-    const int nb = N / R, H = (R - 1) / 2, l = threadIdx.x % LN;
+    const int nb = N / R, H = (R - 1) / 2, l = threadIdx.x % LN, nq = (H + F2_TB) / F2_TB;
     for (int n = threadIdx.x / LN; n < N; n += blockDim.x / LN) f2sm[ia + n * P + l] = ld(n);
     __syncthreads();
-    for (int o = threadIdx.x / LN; o < (H + 1) * nb; o += blockDim.x / LN) {
-        const int t = o / nb, j = o - t * nb;
-        const float2* a = f2sm + ia + j * P + l;
-        float2 e = a[0], d = make_float2(0.f, 0.f);
-        for (int q = 1, i = t; q <= H; ++q) {
-            const float2 x = a[q * nb * P], y = a[(R - q) * nb * P], w = tw[i * nb];
-            e.x = fmaf(x.x + y.x, w.x, e.x);
-            e.y = fmaf(x.y + y.y, w.x, e.y);
-            d.x = fmaf(x.x - y.x, w.y, d.x);
-            d.y = fmaf(x.y - y.y, w.y, d.y);
-            i += t;
-            if (i >= R) i -= R;
+    for (int o = threadIdx.x / LN; o < nq * nb; o += blockDim.x / LN) {
+        const int t0 = o / nb, j = o - t0 * nb, st = nb * P;
+        const float2 *a = f2sm + ia + j * P + l, *xq = a + st, *yq = a + (R - 1) * st, *w = tw + N + t0;
+        float2 e[F2_TB], d[F2_TB];
+        int to[F2_TB];                                       // t values past H repeat t = H
+#pragma unroll
+        for (int m = 0; m < F2_TB; ++m) {
+            e[m] = a[0];
+            d[m] = make_float2(0.f, 0.f);
+            to[m] = min(t0 + m * nq, H) - t0;
         }
-        f2sm[ib + (t * nb + j) * P + l] = make_float2(e.x - s * d.y, e.y + s * d.x);
-        if (t > 0) f2sm[ib + ((R - t) * nb + j) * P + l] = make_float2(e.x + s * d.y, e.y - s * d.x);
+#pragma unroll 2
+        for (int q = 1; q <= H; ++q, xq += st, yq -= st, w += H + 1) {
+            const float2 x = *xq, y = *yq, p = cadd(x, y), r = csub(x, y);
+#pragma unroll
+            for (int m = 0; m < F2_TB; ++m) {
+                const float2 c = w[to[m]];
+                e[m].x = fmaf(p.x, c.x, e[m].x);
+                e[m].y = fmaf(p.y, c.x, e[m].y);
+                d[m].x = fmaf(r.x, c.y, d[m].x);
+                d[m].y = fmaf(r.y, c.y, d[m].y);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < F2_TB; ++m) {
+            const int t = t0 + m * nq;
+            if (t > H) break;
+            f2sm[ib + (t * nb + j) * P + l] = make_float2(e[m].x - s * d[m].y, e[m].y + s * d[m].x);
+            if (t > 0) f2sm[ib + ((R - t) * nb + j) * P + l] = make_float2(e[m].x + s * d[m].y, e[m].y - s * d[m].x);
+        }
     }
 }
 
@@ -247,7 +259,8 @@ k_fft2_row_fwd(const float2* __restrict__ x, const MT* __restrict__ maps, const 
     constexpr int P = LN;
     const int N = ax.N, n0 = geo.n[0], n1 = geo.n[1], g0 = geo.g[0];
     float2* tw = f2sm + 2 * N * P;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = ax.tw[i];
+    const int nt = N + fft_axis_extra(ax);
+    for (int i = threadIdx.x; i < nt; i += blockDim.x) tw[i] = ax.tw[i];
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (iter) *iter += 1;
         if (nrm) { nrm[0] = nrm[1]; nrm[1] = 0.0; }
@@ -291,7 +304,8 @@ k_fft2_col(float2* in, float2* out, Geom geo, F2Axis ax, FfConst k) {
     constexpr int P = LN;
     const int N = ax.N, n0 = geo.n[0], g1 = geo.g[1];
     float2* tw = f2sm + 2 * N * P;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = ax.tw[i];
+    const int nt = N + fft_axis_extra(ax);
+    for (int i = threadIdx.x; i < nt; i += blockDim.x) tw[i] = ax.tw[i];
     const int xblocks = (g1 + LN - 1) / LN;
     const int xb = blockIdx.x % xblocks, c = blockIdx.x / xblocks;
     const int xx = xb * LN + threadIdx.x % LN;
@@ -333,9 +347,10 @@ k_fft2_row_inv(const float2* __restrict__ in, const MT* __restrict__ maps, const
     constexpr int P = LN + 1;                              // the combine reads a point's lines one after another
     const int N = ax.N, n0 = geo.n[0], n1 = geo.n[1], g0 = geo.g[0], C = geo.C;
     float2* tw = f2sm + 2 * N * P;
-    float2* acc = tw + N;                                  // [RW][n1]
+    float2* acc = tw + N + fft_axis_extra(ax);             // [RW][n1]
     const int CS = C < LN ? C : LN, RW = LN / CS;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) tw[i] = ax.tw[i];
+    const int nt = N + fft_axis_extra(ax);
+    for (int i = threadIdx.x; i < nt; i += blockDim.x) tw[i] = ax.tw[i];
     const int l = threadIdx.x % LN, r = l / CS, ci = l - r * CS;
     const int row0 = blockIdx.x * RW, nr = min(RW, n0 - row0), h1 = n1 / 2;
     const int ny = row0 + r - n0 / 2;
@@ -427,21 +442,99 @@ k_fft2_row_inv(const float2* __restrict__ in, const MT* __restrict__ maps, const
     }
 }
 
+// ---------------------------------------------------------------- 3D
+// One pass along AXIS (0 = z, 1 = y, 2 = x) of every coil's 3D grid, for lengths without a compiled
+// pass (kp_fft.cu, whose lines and pruning it follows: forward reads only the image band, inverse
+// writes only it; x passes take only the rows of the band, y passes its planes).  In place for the y,
+// z and inverse passes: a CTA's loads are all in the first stage, before a barrier.
+template <int AXIS, bool INV, bool PRE, typename MT>
+__global__ void __launch_bounds__(F2_T, 4) k_fftg_pass(const float2* in, float2* out, Geom geo, F2Axis ax, FfConst k, PreSrc pre) {
+    constexpr int LN = 8, P = LN;
+    const int N = ax.N, n0 = geo.n[0], n1 = geo.n[1], n2 = geo.n[2], g0 = geo.g[0], g1 = geo.g[1], g2 = geo.g[2];
+    float2* tw = f2sm + 2 * N * P;
+    const int nt = N + fft_axis_extra(ax);
+    for (int i = threadIdx.x; i < nt; i += blockDim.x) tw[i] = ax.tw[i];
+    const int l = threadIdx.x % LN, na = AXIS == 0 ? n0 : AXIS == 1 ? n1 : n2;
+    const int64_t lim = (int64_t)geo.C * geo.G;
+    int64_t base = 0, img = 0;                              // element 0 of this thread's line; its image row
+    int stride = 1, c = 0;
+    float ay = 1.f;
+    bool live;
+    if (AXIS == 2) {
+        const int64_t line = (int64_t)blockIdx.x * LN + l;  // (image row, coil), coil fastest
+        live = line < (int64_t)geo.C * n0 * n1;
+        const int rem = live ? (int)(line / geo.C) : 0;
+        c = live ? (int)(line % geo.C) : 0;
+        const int z = band_index(rem / n1, n0, g0), y = band_index(rem % n1, n1, g1);
+        base = (int64_t)c * geo.G + ((int64_t)z * g1 + y) * g2;
+        if (PRE) {
+            const int pz = pix_index(z, n0, g0), py = pix_index(y, n1, g1);
+            img = ((int64_t)pz * n1 + py) * n2;
+            ay = pre.apod[pz] * pre.apod[n0 + py];
+        }
+    } else {
+        const int xblocks = (g2 + LN - 1) / LN, outer = AXIS == 1 ? n0 : g1;
+        const int xb = blockIdx.x % xblocks, rest = blockIdx.x / xblocks, o = rest % outer;
+        const int x = xb * LN + l;
+        live = x < g2;
+        base = (int64_t)(rest / outer) * geo.G + (AXIS == 1 ? (int64_t)band_index(o, n0, g0) * g1 * g2 : (int64_t)o * g2) + (live ? x : 0);
+        stride = AXIS == 1 ? g2 : g1 * g2;                   // n stride < G < 2^31
+    }
+    const float2* pi = in + base;
+    float2* po = out + base;
+    const float* ax2 = PRE ? pre.apod + n0 + n1 : nullptr;
+    const float2* xr = pre.x + img;
+    const MT* mr = PRE && pre.maps ? (const MT*)pre.maps + (size_t)c * geo.N + img : nullptr;
+    __syncthreads();
+    const float s = INV ? -1.f : 1.f;
+    const int f = f2_begin<LN, P>(ax, [&](int n) {
+        const bool ok = live && (INV || in_band(n, na, N));
+        if constexpr (PRE) {                                // no branches around the loads (see k_fft2_row_fwd)
+            const int px = ok ? pix_index(n, n2, N) : 0;
+            if (!KP_INB(3, px, n2)) return make_float2(0.f, 0.f);
+            float2 v = xr[px];
+            const float2 m = mr ? ldc<MT>(mr, px) : make_float2(1.f, 0.f);
+            const float a = ok ? ay * ax2[px] : 0.f;
+            v.x *= a;
+            v.y *= a;
+            if (mr) v = cmul(m, v);
+            return ok ? v : make_float2(0.f, 0.f);
+        } else {
+            return ok && KP_INB(1, base + (int64_t)n * stride, lim) ? pi[n * stride] : make_float2(0.f, 0.f);
+        }
+    }, N * P, tw, s, k);
+    f2_end<LN, P>(ax, [&](int n, float2 v) {
+        if (live && (!INV || in_band(n, na, N)) && KP_INB(2, base + (int64_t)n * stride, lim)) po[n * stride] = v;
+    }, f, tw, s, k);
+}
+
 // ---------------------------------------------------------------- host
-static size_t fwd_smem(int N, int ln) { return (size_t)(2 * ln + 1) * N * sizeof(float2); }
-static size_t inv_smem(int N, int ln, int acc) { return ((size_t)(2 * (ln + 1) + 1) * N + acc) * sizeof(float2); }
+static size_t fwd_smem(const F2Axis& ax, int ln) { return ((size_t)(2 * ln + 1) * ax.N + fft_axis_extra(ax)) * sizeof(float2); }
+static size_t inv_smem(const F2Axis& ax, int ln, int acc) { return fwd_smem(ax, ln) + ((size_t)2 * ax.N + acc) * sizeof(float2); }
+
+void fft_axis_table(const F2Axis& ax, std::vector<float2>& h) {
+    const auto root = [](int m, int n) {
+        const double a = -2.0 * M_PI * (double)m / (double)n;
+        return make_float2((float)std::cos(a), (float)std::sin(a));
+    };
+    for (int m = 0; m < ax.N; ++m) h.push_back(root(m, ax.N));
+    const int R = ax.r[0], H = (R - 1) / 2;
+    if (fft_axis_extra(ax) > 0)
+        for (int q = 1; q <= H; ++q)
+            for (int t = 0; t <= H; ++t) h.push_back(root(q * t % R, R));
+}
 
 // Threads of a pass: its largest stage in as few equal rounds as F2_T threads allow.
 static int pass_threads(const F2Axis& ax, int ln) {
     int items = 0;
-    for (int i = 0; i < ax.nst; ++i) items = std::max(items, ax.N / (ax.r[i] > 19 ? 2 : ax.r[i]) * ln);
+    for (int i = 0; i < ax.nst; ++i) items = std::max(items, ax.N / (ax.r[i] > 19 ? 2 * F2_TB : ax.r[i]) * ln);
     const int rounds = (items + F2_T - 1) / F2_T;
     return ((items + rounds - 1) / rounds + 31) / 32 * 32;
 }
 
 // Radices of N: at most one prime above 5 (first), then the fewest radices (and the smallest sum)
 // for the rest, at least two in all; false if N is not handled.
-static bool f2_factor(int N, F2Axis& ax) {
+bool fft_axis_factor(int N, F2Axis& ax) {
     static const int rad[] = {10, 9, 8, 6, 5, 4, 3, 2};
     int rest = N;
     std::vector<int> r;
@@ -498,23 +591,21 @@ kp_status fft2_create(kp_plan p) {
     if (env && std::string(env) == "cufft") return KP_OK;
     Fft2Plan f{};
     for (int d = 0; d < 2; ++d)
-        if (!f2_factor(g.g[d], f.ax[d])) return KP_OK;
-    if (inv_smem(g.g[1], 4, g.n[1] * 4) > (size_t)F2_SMEM || fwd_smem(g.g[0], 4) > (size_t)F2_SMEM) return KP_OK;
+        if (!fft_axis_factor(g.g[d], f.ax[d])) return KP_OK;
+    if (inv_smem(f.ax[1], 4, g.n[1] * 4) > (size_t)F2_SMEM || fwd_smem(f.ax[0], 4) > (size_t)F2_SMEM) return KP_OK;
     Fft2Plan* q = new (std::nothrow) Fft2Plan(f);
     if (!q) { set_error("host allocation failed"); return KP_ENOMEM; }
     std::vector<float2> h;
-    for (int d = 0; d < 2; ++d)
-        for (int m = 0; m < g.g[d]; ++m) {
-            const double a = -2.0 * M_PI * (double)m / (double)g.g[d];
-            h.push_back(make_float2((float)std::cos(a), (float)std::sin(a)));
-        }
+    fft_axis_table(f.ax[0], h);
+    const size_t first = h.size();
+    fft_axis_table(f.ax[1], h);
     if (cudaMalloc(&q->d_tw, h.size() * sizeof(float2)) != cudaSuccess) {
         delete q;
         set_error("device allocation failed");
         return KP_ENOMEM;
     }
     q->ax[0].tw = q->d_tw;
-    q->ax[1].tw = q->d_tw + g.g[0];
+    q->ax[1].tw = q->d_tw + first;
     q->k = ff_const();
     p->fft2 = q;
     KP_TRY_CUDA(cudaMemcpy(q->d_tw, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice));
@@ -534,7 +625,7 @@ template <typename MT, int LN>
 static kp_status launch_row_fwd(kp_plan p, const float2* x, int* iter, double* nrm, cudaStream_t st) {
     static SmemLimit lim;
     const Geom& g = p->geo;
-    const size_t sm = fwd_smem(g.g[1], LN);
+    const size_t sm = fwd_smem(p->fft2->ax[1], LN);
     KP_TRY_CUDA(lim.ensure(k_fft2_row_fwd<MT, LN>, sm));
     const unsigned nb = (unsigned)(((int64_t)g.n[0] * g.C + LN - 1) / LN);
     k_fft2_row_fwd<MT, LN><<<nb, pass_threads(p->fft2->ax[1], LN), sm, st>>>(x, p->unit_maps ? nullptr : (const MT*)p->d_maps, p->d_apod, g,
@@ -547,7 +638,7 @@ template <bool INV, int LN>
 static kp_status launch_col(kp_plan p, float2* in, float2* out, cudaStream_t st) {
     static SmemLimit lim;
     const Geom& g = p->geo;
-    const size_t sm = fwd_smem(g.g[0], LN);
+    const size_t sm = fwd_smem(p->fft2->ax[0], LN);
     KP_TRY_CUDA(lim.ensure(k_fft2_col<INV, LN>, sm));
     const unsigned nb = (unsigned)((int64_t)g.C * ((g.g[1] + LN - 1) / LN));
     k_fft2_col<INV, LN><<<nb, pass_threads(p->fft2->ax[0], LN), sm, st>>>(in, out, g, p->fft2->ax[0], p->fft2->k);
@@ -559,7 +650,7 @@ template <bool INV>
 static kp_status col_pass(kp_plan p, float2* in, float2* out, cudaStream_t st) {
     const Geom& g = p->geo;
     p->launches += 1;
-    if (lines_for((int64_t)g.C * ((g.g[1] + 7) / 8), fwd_smem(g.g[0], 8)) == 8) return launch_col<INV, 8>(p, in, out, st);
+    if (lines_for((int64_t)g.C * ((g.g[1] + 7) / 8), fwd_smem(p->fft2->ax[0], 8)) == 8) return launch_col<INV, 8>(p, in, out, st);
     return launch_col<INV, 4>(p, in, out, st);
 }
 
@@ -568,7 +659,7 @@ static kp_status launch_row_inv(kp_plan p, int mode, const F2Step& sp, cudaStrea
     static SmemLimit lim;
     const Geom& g = p->geo;
     const int rw = LN / std::min(g.C, LN);
-    const size_t sm = inv_smem(g.g[1], LN, rw * g.n[1]);
+    const size_t sm = inv_smem(p->fft2->ax[1], LN, rw * g.n[1]);
     KP_TRY_CUDA(lim.ensure(k_fft2_row_inv<MT, LN>, sm));
     const unsigned nb = (unsigned)((g.n[0] + rw - 1) / rw);
     k_fft2_row_inv<MT, LN><<<nb, pass_threads(p->fft2->ax[1], LN), sm, st>>>(
@@ -582,7 +673,7 @@ static kp_status row_inv_t(kp_plan p, int mode, const F2Step& sp, cudaStream_t s
     const Geom& g = p->geo;
     const int rw = 8 / std::min(g.C, 8);
     // 4 lines for up to 4 coils: one image row each without idle lines
-    if (g.C > 4 && lines_for((g.n[0] + rw - 1) / rw, inv_smem(g.g[1], 8, rw * g.n[1])) == 8)
+    if (g.C > 4 && lines_for((g.n[0] + rw - 1) / rw, inv_smem(p->fft2->ax[1], 8, rw * g.n[1])) == 8)
         return launch_row_inv<MT, 8>(p, mode, sp, st);
     return launch_row_inv<MT, 4>(p, mode, sp, st);
 }
@@ -599,7 +690,7 @@ static kp_status row_inv(kp_plan p, int mode, const F2Step& sp, cudaStream_t st)
 template <typename MT>
 static kp_status row_fwd_t(kp_plan p, const float2* x, int* iter, double* nrm, cudaStream_t st) {
     const Geom& g = p->geo;
-    if (lines_for(((int64_t)g.n[0] * g.C + 7) / 8, fwd_smem(g.g[1], 8)) == 8)
+    if (lines_for(((int64_t)g.n[0] * g.C + 7) / 8, fwd_smem(p->fft2->ax[1], 8)) == 8)
         return launch_row_fwd<MT, 8>(p, x, iter, nrm, st);
     return launch_row_fwd<MT, 4>(p, x, iter, nrm, st);
 }
@@ -634,5 +725,32 @@ kp_status fft2_adjoint_primal(kp_plan p, int reg, float lambda, cudaStream_t st)
     sp.lambda = lambda;
     return row_inv(p, reg == KP_REG_L2 ? F2_L2 : reg == KP_REG_TV ? F2_TV : F2_Z, sp, st);
 }
+
+bool fftg_fits(const F2Axis& ax) { return fwd_smem(ax, 8) <= (size_t)F2_SMEM; }
+
+template <int AXIS, bool INV, bool PRE, typename MT>
+kp_status fftg_pass(const F2Axis& ax, const FfConst& k, const Geom& g, const float2* in, float2* out, const PreSrc& pre, cudaStream_t st) {
+    static SmemLimit lim;
+    const size_t sm = fwd_smem(ax, 8);
+    KP_TRY_CUDA(lim.ensure(k_fftg_pass<AXIS, INV, PRE, MT>, sm));
+    const int64_t xblocks = (g.g[2] + 7) / 8;
+    const int64_t nb = AXIS == 2 ? ((int64_t)g.C * g.n[0] * g.n[1] + 7) / 8 : (int64_t)g.C * (AXIS == 1 ? g.n[0] : g.g[1]) * xblocks;
+    if (nb > INT32_MAX) { set_error("grid too large for the FFT passes"); return KP_EINVAL; }
+    k_fftg_pass<AXIS, INV, PRE, MT><<<(unsigned)nb, pass_threads(ax, 8), sm, st>>>(in, out, g, ax, k, pre);
+    KP_LAUNCH_CHECK();
+    return KP_OK;
+}
+#define KP_FFTG(A, I, P, T) \
+    template kp_status fftg_pass<A, I, P, T>(const F2Axis&, const FfConst&, const Geom&, const float2*, float2*, const PreSrc&, cudaStream_t);
+KP_FFTG(2, false, true, float2)
+KP_FFTG(2, false, true, __nv_bfloat162)
+KP_FFTG(2, false, true, __half2)
+KP_FFTG(2, false, false, float2)
+KP_FFTG(1, false, false, float2)
+KP_FFTG(0, false, false, float2)
+KP_FFTG(0, true, false, float2)
+KP_FFTG(1, true, false, float2)
+KP_FFTG(2, true, false, float2)
+#undef KP_FFTG
 
 }  // namespace kp

@@ -5,8 +5,28 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <vector>
 
 namespace kp {
+
+// An axis for the passes of run-time length (kp_fft2.cu).
+constexpr int F2_MAXST = 8;       // radix stages at most
+struct F2Axis {
+    int N, nst;                   // at least two stages
+    int r[F2_MAXST];              // radices in the order applied
+    unsigned mg[F2_MAXST];        // 2^32 / m + 1 for the stage's m (bf / m by a high product)
+    const float2* tw;             // e^{-2 pi i m / N}, then the first radix's table when it is summed directly
+};
+// Radices of N into ax (not tw); false if N is not handled.
+bool fft_axis_factor(int N, F2Axis& ax);
+// Points of the table that the directly summed first radix needs beside the N roots: w_R^(q t), q = 1 ..
+// (R - 1) / 2 by rows, t = 0 .. (R - 1) / 2; 0 for a compiled radix.
+__host__ __device__ inline int fft_axis_extra(const F2Axis& ax) {
+    const int h = (ax.r[0] - 1) / 2;
+    return ax.r[0] > 19 ? h * (h + 1) : 0;
+}
+// The axis's table (float64, rounded once) appended to h; ax.tw is to point at it on the device.
+void fft_axis_table(const F2Axis& ax, std::vector<float2>& h);
 
 struct FfConst {                 // float64 on the host, rounded once
     float s3, c51, s51, c52, s52;   // sqrt(3)/2, cos and sin of 2 pi/5 and of 4 pi/5
@@ -24,6 +44,14 @@ inline FfConst ff_const() {
         k.w16[j] = make_float2((float)std::cos(2.0 * M_PI * j / 16.0), (float)std::sin(2.0 * M_PI * j / 16.0));
     return k;
 }
+
+// The image samples a first forward pass forms itself (coil multiply and apodisation, the
+// NUFFT's pre-step fused into the FFT): x, the maps (null: unit maps) and 1/Phi per axis.
+struct PreSrc {
+    const float2* x;
+    const void* maps;
+    const float* apod;
+};
 
 __device__ __forceinline__ bool in_band(int i, int n, int g) { return i < n - n / 2 || i >= g - n / 2; }
 // pixel index of grid index i (i in the band)

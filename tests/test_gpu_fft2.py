@@ -42,3 +42,28 @@ def test_own_2d_fft(shape, C, alpha, kind):
         xs = plan.pdhg_solve(to_dev(y), to_dev(p), reg, 0.1, 3, lmax=L)[0].cpu().numpy()
         assert rel(xs, ref, reg) < 1e-5
     plan.close()
+
+
+# grids 26x34x22 (2 13, 2 17, 2 11), 94x38x46 (47, 19, 23), 10x62x90 (31), 60x28x166 (compiled, 7, 83), 14x254x12 (7, 127),
+# 48x54x50 (no prime above 5)
+@pytest.mark.parametrize("shape,C,kind", [((20, 27, 17), 3, "c64"), ((75, 30, 36), 1, "fp16"), ((8, 49, 72), 8, "c64"),
+                                          ((48, 22, 132), 5, "bf16"), ((11, 203, 9), 2, "c64"), ((38, 43, 40), 9, "c64")])
+def test_own_3d_fft_of_any_length(shape, C, kind):
+    """The 3D passes of run-time length: forward, adjoint and preconditioner (its 2N grids)."""
+    need_gpu()
+    import torch
+    from oracle import precond as opc
+    from paper_1902_09657_gb300.api import to_storage
+    M = 1200
+    x, maps, traj = random_problem(shape, C, M, seed=C, edge=True)
+    rng = np.random.default_rng(C)
+    y = (rng.standard_normal((C, M)) + 1j * rng.standard_normal((C, M))).astype(np.complex64)
+    md = to_storage(torch.from_numpy(maps).cuda(), kind)
+    m = rounded(md)
+    plan = make_plan(shape, C, M)
+    plan.set_trajectory(to_dev(traj)).set_maps(md)
+    assert rel(plan.sense_forward(to_dev(x)).cpu().numpy(), onf.nufft_forward(x.astype(np.complex128), m, traj), "forward") < 1e-5
+    assert rel(plan.sense_adjoint(to_dev(y)).cpu().numpy(), onf.nufft_adjoint(y.astype(np.complex128), m, traj), "adjoint") < 1e-5
+    if C <= 3:
+        assert rel(plan.make_preconditioner().cpu().numpy(), opc.mc_precond_fast(m, traj), "preconditioner") < 1e-5
+    plan.close()
