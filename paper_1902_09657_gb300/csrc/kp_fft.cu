@@ -411,7 +411,7 @@ void fft3_destroy(kp_plan p) {
 
 // Grid sizes with compiled passes (the 3D workloads' grids and their preconditioner's 2N grids,
 // and small test grids); another length takes the passes of run-time length (150 x 132 x 116 x 5 coils,
-// grid 188 x 166 x 146 with the primes 47, 83 and 73: @@G).
+// grid 188 x 166 x 146 with the primes 47, 83 and 73: adjoint 1.33 ms, with cuFFT 1.79 ms).
 #define KP_FFT_SIZES(X) X(20) X(30) X(40) X(60) X(80) X(100) X(120) X(160) X(200) X(240) X(320) X(384) X(400) X(480)
 
 static bool size_compiled(int N) {

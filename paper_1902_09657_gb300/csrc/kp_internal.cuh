@@ -481,6 +481,8 @@ struct kp_plan_s {
     size_t tape_cap = 0;
     int tape_iters = 0;
     float tape_lambda = 0.f;
+    float* d_dwt = nullptr;          // [D * W][M] Kaiser-Bessel derivatives per sorted sample (trajectory gradients)
+    int dwt_version = -1;            // traj_version they belong to
     float2* d_bk = nullptr;          // [2][C][M] reverse-sweep k-space work (g_r, g_y)
 
     kp::Graph graphs[3];             // per regulariser

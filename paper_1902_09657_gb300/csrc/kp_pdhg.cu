@@ -158,43 +158,45 @@ __global__ void k_norm2_clear(const float2* __restrict__ x, int64_t n, double* _
 __global__ void k_store_sqrt(const double* __restrict__ n2, double* __restrict__ out) { *out = sqrt(*n2); }
 
 // Step sizes (Sec. 4.1): sigma_0 = 1, tau_0 = 1/L, theta_k = 1/(1 + 2 sigma_k pmin),
-// sigma_{k+1} = theta_k sigma_k, tau_{k+1} = tau_k / theta_k; float64 recursion.
+// sigma_{k+1} = theta_k sigma_k, tau_{k+1} = tau_k / theta_k, in float64.  The recursion has the
+// closed form 1/sigma_{k+1} = 1/sigma_k + 2 pmin, so sigma_k = 1/(1 + 2 k pmin) and tau_k = 1/(L sigma_k),
+// and every k is independent (one thread's recursion took 0.7 us per iteration, 69 us for 100).
 // schedd: [0] L, [1] pmin (written here from minbits), [2] sigma_last, [3] tau_last.
 // tv_d > 0: the fixed steps of Sec. 4.2 for TV in tv_d dimensions, sigma = theta = 1 and
-// tau = 1/(L + lambda_max(G G^H)) with lambda_max(G G^H) = 4 tv_d.
+// tau = 1/(L + lambda_max(G G^H)) with lambda_max(G G^H) = 4 tv_d.  One CTA.
 __global__ void k_schedule(double* __restrict__ schedd, const int* __restrict__ minbits, int iters,
                            float* __restrict__ sched, int* __restrict__ flag, int tv_d) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const double L = schedd[0];
     const double pmin = minbits ? (double)__int_as_float(*minbits) : schedd[1];
-    schedd[1] = pmin;
-    if (!(L > 0) || !isfinite(L) || !(pmin > 0) || !isfinite(pmin)) {
-        flag[0] = 1;
-        for (int k = 0; k < iters; ++k) { sched[3 * k] = 0.f; sched[3 * k + 1] = 0.f; sched[3 * k + 2] = 0.f; }
-        return;
-    }
-    if (tv_d > 0) {
-        const double tau = 1.0 / (L + 4.0 * tv_d);
-        for (int k = 0; k < iters; ++k) {
-            sched[3 * k] = 1.f;
-            sched[3 * k + 1] = (float)tau;
-            sched[3 * k + 2] = 1.f;
+    __syncthreads();                                       // schedd has been read
+    const bool bad = !(L > 0) || !isfinite(L) || !(pmin > 0) || !isfinite(pmin);
+    for (int k = threadIdx.x; k < iters; k += blockDim.x) {
+        double sig = 0.0, tau = 0.0, th = 0.0;
+        if (!bad && tv_d > 0) {
+            sig = th = 1.0;
+            tau = 1.0 / (L + 4.0 * tv_d);
+        } else if (!bad) {
+            const double r = 1.0 + 2.0 * pmin * k;         // 1 / sigma_k
+            sig = 1.0 / r;
+            tau = r / L;
+            th = r / (r + 2.0 * pmin);
         }
-        schedd[2] = 1.0;
-        schedd[3] = tau;
-        return;
-    }
-    double sig = 1.0, tau = 1.0 / L;
-    for (int k = 0; k < iters; ++k) {
-        const double th = 1.0 / (1.0 + 2.0 * sig * pmin);
         sched[3 * k] = (float)sig;
         sched[3 * k + 1] = (float)tau;
         sched[3 * k + 2] = (float)th;
-        sig *= th;
-        tau /= th;
     }
-    schedd[2] = sig;
-    schedd[3] = tau;
+    if (threadIdx.x != 0) return;
+    schedd[1] = pmin;
+    if (bad) {
+        flag[0] = 1;
+    } else if (tv_d > 0) {
+        schedd[2] = 1.0;
+        schedd[3] = 1.0 / (L + 4.0 * tv_d);
+    } else {
+        const double r = 1.0 + 2.0 * pmin * iters;
+        schedd[2] = 1.0 / r;
+        schedd[3] = r / L;
+    }
 }
 
 __global__ void k_advance(int* iter) { *iter += 1; }
@@ -488,7 +490,7 @@ kp_status solve_setup_b(kp_plan plan, int iters, cudaStream_t st, int reg, const
     const Geom& g = plan->geo;
     const int k0 = start ? start->k : 0;
     iters += k0;                       // the schedule runs from iteration 0; the run starts at k0
-    k_schedule<<<1, 1, 0, st>>>(plan->d_schedd, plan->d_flag + 4, std::max(iters, 1), plan->d_sched, plan->d_flag + 6,
+    k_schedule<<<1, 128, 0, st>>>(plan->d_schedd, plan->d_flag + 4, std::max(iters, 1), plan->d_sched, plan->d_flag + 6,
                                 reg == KP_REG_TV ? g.D : 0);
     KP_LAUNCH_CHECK();
     plan->launches += 1;
