@@ -163,7 +163,8 @@ kp_status kp_max_eig(kp_plan plan, const float* p_dev, const void* v0_dev, int i
  *   v <- projection of v + sigma G xbar onto {|v_i| <= lambda},
  *   x <- x - tau (A^H u + G^H v),  xbar <- 2 x - x_old,
  * with sigma = 1, theta = 1 and tau = 1/(lmax + 4 ndim) at every iteration, v_0 = 0.
- * The iteration is replayed from a CUDA graph captured once per plan and regulariser.
+ * The iteration is replayed from a CUDA graph captured once per plan and regulariser (2D plans on
+ * the own FFT issue its kernels directly, linked by programmatic launches).
  * Synchronous.  Errors: KP_EINVAL (iters < 0, lambda < 0, wavelet levels 0 for l1,
  * non-positive p or lmax found on the device), KP_ENONFINITE (the returned x holds a NaN or
  * Inf, checked on the device after every solve, or a non-finite objective in the trace),

@@ -261,6 +261,7 @@ k_fft2_row_fwd(const float2* __restrict__ x, const MT* __restrict__ maps, const 
     float2* tw = f2sm + 2 * N * P;
     const int nt = N + fft_axis_extra(ax);
     for (int i = threadIdx.x; i < nt; i += blockDim.x) tw[i] = ax.tw[i];
+    pdl_begin();                                           // (the tables above are constant)
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (iter) *iter += 1;
         if (nrm) { nrm[0] = nrm[1]; nrm[1] = 0.0; }
@@ -311,6 +312,7 @@ k_fft2_col(float2* in, float2* out, Geom geo, F2Axis ax, FfConst k) {
     const int xx = xb * LN + threadIdx.x % LN;
     const bool live = xx < g1;
     const int64_t base = (int64_t)c * geo.G + xx, lim = (int64_t)geo.C * geo.G;
+    pdl_begin();
     __syncthreads();
     float2* pi = in + base;                                // n g1 < G < 2^31
     float2* po = out + base;
@@ -354,6 +356,7 @@ k_fft2_row_inv(const float2* __restrict__ in, const MT* __restrict__ maps, const
     const int l = threadIdx.x % LN, r = l / CS, ci = l - r * CS;
     const int row0 = blockIdx.x * RW, nr = min(RW, n0 - row0), h1 = n1 / 2;
     const int ny = row0 + r - n0 / 2;
+    pdl_begin();
     __syncthreads();
     for (int c0 = 0; c0 < C; c0 += CS) {
         const int cc = min(CS, C - c0);
@@ -628,9 +631,9 @@ static kp_status launch_row_fwd(kp_plan p, const float2* x, int* iter, double* n
     const size_t sm = fwd_smem(p->fft2->ax[1], LN);
     KP_TRY_CUDA(lim.ensure(k_fft2_row_fwd<MT, LN>, sm));
     const unsigned nb = (unsigned)(((int64_t)g.n[0] * g.C + LN - 1) / LN);
-    k_fft2_row_fwd<MT, LN><<<nb, pass_threads(p->fft2->ax[1], LN), sm, st>>>(x, p->unit_maps ? nullptr : (const MT*)p->d_maps, p->d_apod, g,
-                                                    p->fft2->ax[1], p->fft2->k, p->d_gridF, iter, nrm);
-    KP_LAUNCH_CHECK();
+    KP_TRY_CUDA(launch_pdl(k_fft2_row_fwd<MT, LN>, nb, pass_threads(p->fft2->ax[1], LN), sm, st, x,
+                           p->unit_maps ? nullptr : (const MT*)p->d_maps, p->d_apod, g, p->fft2->ax[1], p->fft2->k,
+                           p->d_gridF, iter, nrm));
     return KP_OK;
 }
 
@@ -641,8 +644,7 @@ static kp_status launch_col(kp_plan p, float2* in, float2* out, cudaStream_t st)
     const size_t sm = fwd_smem(p->fft2->ax[0], LN);
     KP_TRY_CUDA(lim.ensure(k_fft2_col<INV, LN>, sm));
     const unsigned nb = (unsigned)((int64_t)g.C * ((g.g[1] + LN - 1) / LN));
-    k_fft2_col<INV, LN><<<nb, pass_threads(p->fft2->ax[0], LN), sm, st>>>(in, out, g, p->fft2->ax[0], p->fft2->k);
-    KP_LAUNCH_CHECK();
+    KP_TRY_CUDA(launch_pdl(k_fft2_col<INV, LN>, nb, pass_threads(p->fft2->ax[0], LN), sm, st, in, out, g, p->fft2->ax[0], p->fft2->k));
     return KP_OK;
 }
 
@@ -662,9 +664,8 @@ static kp_status launch_row_inv(kp_plan p, int mode, const F2Step& sp, cudaStrea
     const size_t sm = inv_smem(p->fft2->ax[1], LN, rw * g.n[1]);
     KP_TRY_CUDA(lim.ensure(k_fft2_row_inv<MT, LN>, sm));
     const unsigned nb = (unsigned)((g.n[0] + rw - 1) / rw);
-    k_fft2_row_inv<MT, LN><<<nb, pass_threads(p->fft2->ax[1], LN), sm, st>>>(
-        p->d_grid, p->unit_maps ? nullptr : (const MT*)p->d_maps, p->d_apod, g, p->fft2->ax[1], p->fft2->k, mode, sp);
-    KP_LAUNCH_CHECK();
+    KP_TRY_CUDA(launch_pdl(k_fft2_row_inv<MT, LN>, nb, pass_threads(p->fft2->ax[1], LN), sm, st, p->d_grid,
+                           p->unit_maps ? nullptr : (const MT*)p->d_maps, p->d_apod, g, p->fft2->ax[1], p->fft2->k, mode, sp));
     return KP_OK;
 }
 

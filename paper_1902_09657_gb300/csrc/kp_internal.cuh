@@ -188,6 +188,33 @@ __device__ __forceinline__ ff32 ff_add(ff32 x, ff32 y) {
 }
 __device__ __forceinline__ double ff_to_double(ff32 x) { return (double)x.hi + (double)x.lo; }
 
+// Programmatic dependent launch of the 2D iteration's kernels: launch_pdl lets a kernel be made ready
+// while the one before it runs, so that its blocks start as that one's exit, and pdl_begin() (at the
+// top of every such kernel, by all threads, before it touches anything another kernel writes) waits
+// until that kernel has completed and its writes are visible.  Each kernel waits before it can
+// complete, so completion is transitive along the chain.  An ordinary launch before or after orders
+// as usual.  The chains are 3 to 7 kernels of 5 to 17 us: adjoint 256^2 x 12 coils 47.1 -> 39.0 us,
+// forward 217 x 186 x 7 25.7 -> 20.8 us, 128^2 l2 reconstruction 2.90 -> 2.42 ms.  No kernel lets its
+// successor start early (griddepcontrol.launch_dependents): blocks placed while the last ones still
+// run pile up on the SMs that are free, and the TV frame went from 3.16 to 3.62 ms.
+__device__ __forceinline__ void pdl_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... KA, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KA>(args)...);
+}
+
 // Once-per-device flag for host-side set-up that the runtime keeps per device, such as
 // cudaFuncSetAttribute (devices 0..63): first() is true the first time it is asked on the
 // current device.

@@ -464,6 +464,7 @@ template <int D, int MODE, typename T>
 __global__ void __launch_bounds__(IP_THREADS, 4)
 k_interp_tile(const int4* __restrict__ items, const int* __restrict__ k0t, const float* __restrict__ wt,
               const float2* __restrict__ grid, Geom geo, Tiles tl, InterpIO io, int c_first) {
+    pdl_begin();
     interp_tile_body<D, MODE, T>(items, k0t, wt, grid, geo, tl, io, blockIdx.x, c_first + blockIdx.y * IP_CH);
 }
 
@@ -1951,6 +1952,7 @@ __global__ void __launch_bounds__(RS_WARPS * 32)
 k_spread_run(const int* __restrict__ k0t, const float* __restrict__ wt, const UT* __restrict__ u,
              const int* __restrict__ perm, Geom geo, int run, float2* __restrict__ grid) {
     __shared__ __align__(16) unsigned char sm[RS_WARPS * run_warp_smem<8>()];
+    pdl_begin();
     const int warp = threadIdx.x >> 5;
     const int64_t beg = ((int64_t)blockIdx.x * RS_WARPS + warp) * run;
     const int64_t end = beg + run < geo.M ? beg + run : geo.M;
@@ -2316,6 +2318,7 @@ __device__ __forceinline__ void pix_coords(int64_t j, const Geom& geo, int* jj, 
 template <int D>
 __global__ void k_tv_dual(const float2* __restrict__ xbar, float2* __restrict__ v, Geom geo,
                           const float* __restrict__ sched, const int* __restrict__ iter, float lambda) {
+    pdl_begin();
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= geo.N) return;
     const float sigma = sched[3 * (*iter)];
@@ -2503,8 +2506,8 @@ static kp_status launch_interp_tile(kp_plan p, const InterpIO& io, int c_first, 
     const size_t smem = (size_t)std::min(IP_CH, left) * IpL<D>::PER_COIL * sizeof(float2);
     if (D == 2 && p->chunk > IP_THREADS) { set_error("interpolation items larger than the block"); return KP_EINTERNAL; }
     if (attr.first()) KP_TRY_CUDA(cudaFuncSetAttribute(k_interp_tile<D, MODE, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
-    k_interp_tile<D, MODE, T><<<dim3((unsigned)p->n_iitems, (left + IP_CH - 1) / IP_CH), IP_THREADS, smem, st>>>(
-        p->d_iitems, p->d_k0, p->d_wt, p->d_gridF, p->geo, p->tiles, io, c_first);
+    KP_TRY_CUDA(launch_pdl(k_interp_tile<D, MODE, T>, dim3((unsigned)p->n_iitems, (left + IP_CH - 1) / IP_CH), IP_THREADS, smem, st,
+                           p->d_iitems, p->d_k0, p->d_wt, p->d_gridF, p->geo, p->tiles, io, c_first));
     return KP_OK;
 }
 
@@ -2676,8 +2679,8 @@ static kp_status launch_spread_run(kp_plan p, const UT* u, const int* perm, cuda
     if (g.D != 2) { set_error("spreading variant 13 is 2D only"); return KP_EINTERNAL; }
     if (!p->fft2) KP_TRY_CUDA(cudaMemsetAsync(p->d_grid2, 0, (size_t)g.C * g.G * sizeof(float2), st));
     const int run = spread_run_len(g);
-    k_spread_run<UT><<<dim3(nblk(g.M, run * RS_WARPS), (g.C + 7) / 8), RS_WARPS * 32, 0, st>>>(p->d_k0, p->d_wt, u, perm, g,
-                                                                                              run, p->d_grid2);
+    KP_TRY_CUDA(launch_pdl(k_spread_run<UT>, dim3(nblk(g.M, run * RS_WARPS), (g.C + 7) / 8), RS_WARPS * 32, 0, st, p->d_k0, p->d_wt,
+                           u, perm, g, run, p->d_grid2));
     return KP_OK;
 }
 
@@ -2940,8 +2943,7 @@ kp_status adjoint_primal(kp_plan p, int reg, float lambda, cudaStream_t st) {
         if (reg == KP_REG_TV) {
             if (!p->d_v) { set_error("TV dual variable not allocated"); return KP_EINTERNAL; }
             p->launches += 1;
-            k_tv_dual<2><<<nblk(g.N, 256), 256, 0, st>>>(p->d_xbar, p->d_v, g, p->d_sched, p->d_iter, lambda);
-            KP_LAUNCH_CHECK();
+            KP_TRY_CUDA(launch_pdl(k_tv_dual<2>, nblk(g.N, 256), 256, 0, st, p->d_xbar, p->d_v, g, p->d_sched, p->d_iter, lambda));
         }
         return fft2_adjoint_primal(p, reg, lambda, st);
     }

@@ -918,6 +918,7 @@ template <int NC>
 __global__ void __launch_bounds__(CP_THREADS)
 k_wprox_cluster(const float2* __restrict__ z, float2* __restrict__ x, float2* __restrict__ xbar,
                 const float* __restrict__ sched, const int* __restrict__ iter, float lambda, int n0, int n1, int L) {
+    pdl_begin();
     cgc::cluster_group cl = cgc::this_cluster();
     const int r = (int)cl.block_rank();
     extern __shared__ __align__(16) float2 smc[];
@@ -1092,8 +1093,10 @@ static cudaLaunchConfig_t cluster_cfg(size_t sm, cudaStream_t st, cudaLaunchAttr
     at[0].val.clusterDim.x = NC;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // pdl_begin
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cfg;
 }
 
@@ -1111,8 +1114,10 @@ static bool cluster_fits(size_t sm) {
         cudaGetLastError();
         return false;
     }
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     cudaLaunchConfig_t cfg = cluster_cfg<NC>(sm, nullptr, at);
+    cfg.numAttrs = 1;                       // the cluster size alone
+
     int nclusters = 0;
     if (cudaOccupancyMaxActiveClusters(&nclusters, k_wprox_cluster<NC>, &cfg) != cudaSuccess) {
         cudaGetLastError();
@@ -1152,7 +1157,7 @@ kp_status primal_cluster(kp_plan p, float lambda, cudaStream_t st) {
     KP_TRY(adjoint_primal(p, KP_REG_L1_WAVELET, lambda, st));
     mark(p, PH_DWT_FWD, st);
     const size_t sm = cluster_smem(g, nc);
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     if (nc == 16) {
         KP_TRY_CUDA(cluster_limit<16>().ensure(k_wprox_cluster<16>, sm));
         cudaLaunchConfig_t cfg = cluster_cfg<16>(sm, st, at);
