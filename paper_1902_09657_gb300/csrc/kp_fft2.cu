@@ -250,12 +250,15 @@ __device__ __forceinline__ void f2_end(const F2Axis& ax, ST st, int from, const 
     }
 }
 
-// Forward row pass: LN lines (image row, coil), coil fastest.  iter (or null) is advanced and nrm (or
-// null) shifted, nrm[0] = nrm[1], nrm[1] = 0, for the kernels that follow.
-template <typename MT, int LN>
+// Forward row pass: LN lines (image row, coil), coil fastest; coil c takes the image x + c xstride.
+// PAIR: "coil" c is the pair (e, f) = pairs[c] of the preconditioner and its image s_e s_f^* (ones
+// without maps).  iter (or null) is advanced and nrm (or null) shifted, nrm[0] = nrm[1], nrm[1] = 0, for
+// the kernels that follow.
+template <typename MT, int LN, bool PAIR>
 __global__ void __launch_bounds__(F2_T, 4)
-k_fft2_row_fwd(const float2* __restrict__ x, const MT* __restrict__ maps, const float* __restrict__ apod, Geom geo,
-               F2Axis ax, FfConst k, float2* __restrict__ out, int* __restrict__ iter, double* __restrict__ nrm) {
+k_fft2_row_fwd(const float2* __restrict__ x, int64_t xstride, const int2* __restrict__ pairs, const MT* __restrict__ maps,
+               const float* __restrict__ apod, Geom geo, F2Axis ax, FfConst k, float2* __restrict__ out,
+               int* __restrict__ iter, double* __restrict__ nrm) {
     constexpr int P = LN;
     const int N = ax.N, n0 = geo.n[0], n1 = geo.n[1], g0 = geo.g[0];
     float2* tw = f2sm + 2 * N * P;
@@ -270,16 +273,22 @@ k_fft2_row_fwd(const float2* __restrict__ x, const MT* __restrict__ maps, const 
     const bool live = line < n0 * geo.C;
     const int iy = live ? line / geo.C : 0, c = live ? line - iy * geo.C : 0;
     const int ny = iy - n0 / 2;
-    const float ay = apod[iy];
+    const float ay = PAIR ? 1.f : apod[iy];
     const float* ax1 = apod + n0;
-    const float2* xr = x + (size_t)iy * n1;
-    const MT* mr = maps ? maps + (size_t)c * geo.N + (size_t)iy * n1 : nullptr;
+    const float2* xr = x + (PAIR ? 0 : (size_t)c * xstride + (size_t)iy * n1);
+    const int2 ef = PAIR && maps ? pairs[c] : make_int2(c, c);
+    const MT* mr = maps ? maps + (size_t)ef.x * geo.N + (size_t)iy * n1 : nullptr;
+    const MT* mf = PAIR && maps ? maps + (size_t)ef.y * geo.N + (size_t)iy * n1 : nullptr;
     __syncthreads();
     // loads without branches (points outside the band read the row's first pixel and drop it), so
     // that a butterfly's loads are all issued before the first is used
     const auto ld = [&](int n) {
         const bool in = live && in_band(n, n1, N) && KP_INB(3, pix_index(n, n1, N), n1);
         const int px = in ? pix_index(n, n1, N) : 0;
+        if constexpr (PAIR) {
+            const float2 e = maps ? ldc<MT>(mr, px) : make_float2(1.f, 0.f), f = maps ? ldc<MT>(mf, px) : make_float2(1.f, 0.f);
+            return in ? cmulc(f, e) : make_float2(0.f, 0.f);
+        }
         float2 v = xr[px];
         const float2 m = maps ? ldc<MT>(mr, px) : make_float2(1.f, 0.f);
         const float a = in ? ay * ax1[px] : 0.f;
@@ -587,73 +596,113 @@ bool fft_axis_factor(int N, F2Axis& ax) {
 // memory than a CTA has.
 static int lines_for(int64_t blocks8, size_t smem8) { return blocks8 >= 152 && smem8 <= (size_t)F2_SMEM ? 8 : 4; }
 
-kp_status fft2_create(kp_plan p) {
-    const Geom& g = p->geo;
-    if (g.D != 2) return KP_OK;
+// Passes for grids of g0 x g1 points (image rows up to n1 points); null when a length is not handled, or
+// KPDHG_FFT=cufft.  *status tells an allocation failure from that.
+Fft2Plan* fft2_make(int g0, int g1, int n1, kp_status* status) {
+    *status = KP_OK;
     const char* env = std::getenv("KPDHG_FFT");
-    if (env && std::string(env) == "cufft") return KP_OK;
+    if (env && std::string(env) == "cufft") return nullptr;
     Fft2Plan f{};
-    for (int d = 0; d < 2; ++d)
-        if (!fft_axis_factor(g.g[d], f.ax[d])) return KP_OK;
-    if (inv_smem(f.ax[1], 4, g.n[1] * 4) > (size_t)F2_SMEM || fwd_smem(f.ax[0], 4) > (size_t)F2_SMEM) return KP_OK;
+    if (!fft_axis_factor(g0, f.ax[0]) || !fft_axis_factor(g1, f.ax[1])) return nullptr;
+    if (inv_smem(f.ax[1], 4, n1 * 4) > (size_t)F2_SMEM || fwd_smem(f.ax[0], 4) > (size_t)F2_SMEM) return nullptr;
     Fft2Plan* q = new (std::nothrow) Fft2Plan(f);
-    if (!q) { set_error("host allocation failed"); return KP_ENOMEM; }
+    *status = KP_ENOMEM;
+    if (!q) { set_error("host allocation failed"); return nullptr; }
     std::vector<float2> h;
     fft_axis_table(f.ax[0], h);
     const size_t first = h.size();
     fft_axis_table(f.ax[1], h);
-    if (cudaMalloc(&q->d_tw, h.size() * sizeof(float2)) != cudaSuccess) {
-        delete q;
+    if (cudaMalloc(&q->d_tw, h.size() * sizeof(float2)) != cudaSuccess ||
+        cudaMemcpy(q->d_tw, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaGetLastError();
+        fft2_free(q);
         set_error("device allocation failed");
-        return KP_ENOMEM;
+        return nullptr;
     }
+    *status = KP_OK;
     q->ax[0].tw = q->d_tw;
     q->ax[1].tw = q->d_tw + first;
     q->k = ff_const();
-    p->fft2 = q;
-    KP_TRY_CUDA(cudaMemcpy(q->d_tw, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice));
+    return q;
+}
+
+void fft2_free(Fft2Plan* q) {
+    if (!q) return;
+    if (q->d_tw) cudaFree(q->d_tw);
+    delete q;
+}
+
+kp_status fft2_create(kp_plan p) {
+    const Geom& g = p->geo;
+    if (g.D != 2) return KP_OK;
+    kp_status st;
+    p->fft2 = fft2_make(g.g[0], g.g[1], g.n[1], &st);
+    if (!p->fft2) return st;
     // the spread grid is zero between adjoints (the inverse column pass clears what it reads)
     KP_TRY_CUDA(cudaMemset(p->d_grid2, 0, (size_t)g.C * g.G * sizeof(float2)));
     return KP_OK;
 }
 
 void fft2_destroy(kp_plan p) {
-    if (!p->fft2) return;
-    if (p->fft2->d_tw) cudaFree(p->fft2->d_tw);
-    delete p->fft2;
+    fft2_free(p->fft2);
     p->fft2 = nullptr;
 }
 
-template <typename MT, int LN>
-static kp_status launch_row_fwd(kp_plan p, const float2* x, int* iter, double* nrm, cudaStream_t st) {
+// Where a forward transform takes its images from (k_fft2_row_fwd).
+struct F2Src {
+    const float2* x;
+    int64_t xstride;
+    const int2* pairs;
+    bool pair;
+    const void* maps;
+    const float* apod;
+    int* iter;
+    double* nrm;
+};
+
+template <typename MT, int LN, bool PAIR>
+static kp_status launch_row_fwd(const Fft2Plan* f, const Geom& g, const F2Src& a, float2* out, cudaStream_t st) {
     static SmemLimit lim;
-    const Geom& g = p->geo;
-    const size_t sm = fwd_smem(p->fft2->ax[1], LN);
-    KP_TRY_CUDA(lim.ensure(k_fft2_row_fwd<MT, LN>, sm));
+    const size_t sm = fwd_smem(f->ax[1], LN);
+    KP_TRY_CUDA(lim.ensure(k_fft2_row_fwd<MT, LN, PAIR>, sm));
     const unsigned nb = (unsigned)(((int64_t)g.n[0] * g.C + LN - 1) / LN);
-    KP_TRY_CUDA(launch_pdl(k_fft2_row_fwd<MT, LN>, nb, pass_threads(p->fft2->ax[1], LN), sm, st, x,
-                           p->unit_maps ? nullptr : (const MT*)p->d_maps, p->d_apod, g, p->fft2->ax[1], p->fft2->k,
-                           p->d_gridF, iter, nrm));
+    KP_TRY_CUDA(launch_pdl(k_fft2_row_fwd<MT, LN, PAIR>, nb, pass_threads(f->ax[1], LN), sm, st, a.x, a.xstride, a.pairs,
+                           (const MT*)a.maps, a.apod, g, f->ax[1], f->k, out, a.iter, a.nrm));
     return KP_OK;
 }
 
+template <typename MT>
+static kp_status row_fwd_t(const Fft2Plan* f, const Geom& g, const F2Src& a, float2* out, cudaStream_t st) {
+    const bool eight = lines_for(((int64_t)g.n[0] * g.C + 7) / 8, fwd_smem(f->ax[1], 8)) == 8;
+    if (a.pair) return eight ? launch_row_fwd<MT, 8, true>(f, g, a, out, st) : launch_row_fwd<MT, 4, true>(f, g, a, out, st);
+    return eight ? launch_row_fwd<MT, 8, false>(f, g, a, out, st) : launch_row_fwd<MT, 4, false>(f, g, a, out, st);
+}
+
 template <bool INV, int LN>
-static kp_status launch_col(kp_plan p, float2* in, float2* out, cudaStream_t st) {
+static kp_status launch_col(const Fft2Plan* f, const Geom& g, float2* in, float2* out, cudaStream_t st) {
     static SmemLimit lim;
-    const Geom& g = p->geo;
-    const size_t sm = fwd_smem(p->fft2->ax[0], LN);
+    const size_t sm = fwd_smem(f->ax[0], LN);
     KP_TRY_CUDA(lim.ensure(k_fft2_col<INV, LN>, sm));
     const unsigned nb = (unsigned)((int64_t)g.C * ((g.g[1] + LN - 1) / LN));
-    KP_TRY_CUDA(launch_pdl(k_fft2_col<INV, LN>, nb, pass_threads(p->fft2->ax[0], LN), sm, st, in, out, g, p->fft2->ax[0], p->fft2->k));
+    KP_TRY_CUDA(launch_pdl(k_fft2_col<INV, LN>, nb, pass_threads(f->ax[0], LN), sm, st, in, out, g, f->ax[0], f->k));
     return KP_OK;
 }
 
 template <bool INV>
-static kp_status col_pass(kp_plan p, float2* in, float2* out, cudaStream_t st) {
-    const Geom& g = p->geo;
-    p->launches += 1;
-    if (lines_for((int64_t)g.C * ((g.g[1] + 7) / 8), fwd_smem(p->fft2->ax[0], 8)) == 8) return launch_col<INV, 8>(p, in, out, st);
-    return launch_col<INV, 4>(p, in, out, st);
+static kp_status col_pass(const Fft2Plan* f, const Geom& g, float2* in, float2* out, cudaStream_t st) {
+    if (lines_for((int64_t)g.C * ((g.g[1] + 7) / 8), fwd_smem(f->ax[0], 8)) == 8) return launch_col<INV, 8>(f, g, in, out, st);
+    return launch_col<INV, 4>(f, g, in, out, st);
+}
+
+static kp_status forward_src(const Fft2Plan* f, const Geom& g, kp_cdtype mt, const F2Src& a, float2* out, int64_t& launches,
+                             cudaStream_t st) {
+    launches += 2;
+    switch (a.maps ? mt : KP_C64) {
+        case KP_C64: KP_TRY(row_fwd_t<float2>(f, g, a, out, st)); break;
+        case KP_C32_BF16: KP_TRY(row_fwd_t<__nv_bfloat162>(f, g, a, out, st)); break;
+        default: KP_TRY(row_fwd_t<__half2>(f, g, a, out, st)); break;
+    }
+    return col_pass<false>(f, g, out, out, st);
 }
 
 template <typename MT, int LN>
@@ -689,25 +738,28 @@ static kp_status row_inv(kp_plan p, int mode, const F2Step& sp, cudaStream_t st)
     }
 }
 
-template <typename MT>
-static kp_status row_fwd_t(kp_plan p, const float2* x, int* iter, double* nrm, cudaStream_t st) {
-    const Geom& g = p->geo;
-    if (lines_for(((int64_t)g.n[0] * g.C + 7) / 8, fwd_smem(p->fft2->ax[1], 8)) == 8)
-        return launch_row_fwd<MT, 8>(p, x, iter, nrm, st);
-    return launch_row_fwd<MT, 4>(p, x, iter, nrm, st);
-}
-
 kp_status fft2_forward_image(kp_plan p, const float2* x, int* iter, double* nrm, cudaStream_t st) {
-    p->launches += 1;
-    switch (p->unit_maps ? KP_C64 : p->maps_t) {
-        case KP_C64: KP_TRY(row_fwd_t<float2>(p, x, iter, nrm, st)); break;
-        case KP_C32_BF16: KP_TRY(row_fwd_t<__nv_bfloat162>(p, x, iter, nrm, st)); break;
-        default: KP_TRY(row_fwd_t<__half2>(p, x, iter, nrm, st)); break;
-    }
-    return col_pass<false>(p, p->d_gridF, p->d_gridF, st);
+    const F2Src a{x, 0, nullptr, false, p->unit_maps ? nullptr : p->d_maps, p->d_apod, iter, nrm};
+    return forward_src(p->fft2, p->geo, p->maps_t, a, p->d_gridF, p->launches, st);
 }
 
-kp_status fft2_inverse_cols(kp_plan p, cudaStream_t st) { return col_pass<true>(p, p->d_grid2, p->d_grid, st); }
+kp_status fft2_forward_batch(kp_plan p, const float2* x, int n, float2* out, cudaStream_t st) {
+    Geom g = p->geo;
+    g.C = n;
+    const F2Src a{x, g.N, nullptr, false, nullptr, p->d_apod, nullptr, nullptr};
+    return forward_src(p->fft2, g, KP_C64, a, out, p->launches, st);
+}
+
+kp_status fft2_forward_pairs(const Fft2Plan* f, const Geom& g, kp_cdtype mt, const void* maps, const int2* pairs, float2* out,
+                             int64_t& launches, cudaStream_t st) {
+    const F2Src a{nullptr, 0, pairs, true, maps, nullptr, nullptr, nullptr};
+    return forward_src(f, g, mt, a, out, launches, st);
+}
+
+kp_status fft2_inverse_cols(kp_plan p, cudaStream_t st) {
+    p->launches += 1;
+    return col_pass<true>(p->fft2, p->geo, p->d_grid2, p->d_grid, st);
+}
 
 kp_status fft2_adjoint_image(kp_plan p, float2* x, double* nrm, cudaStream_t st) {
     F2Step sp{};

@@ -627,6 +627,13 @@ void fft2_destroy(kp_plan p);
 // The forward grid spectrum of image x into d_gridF (coil multiply and apodisation included).  The
 // first kernel also advances *iter (unless null) and shifts nrm[0] = nrm[1], nrm[1] = 0 (unless null).
 kp_status fft2_forward_image(kp_plan p, const float2* x, int* iter, double* nrm, cudaStream_t st);
+// The same for n images x [n][N] in one go (unit maps), into out [n][G].
+kp_status fft2_forward_batch(kp_plan p, const float2* x, int n, float2* out, cudaStream_t st);
+// Spectra of the zero-padded pair products s_e s_f^* (ones without maps) on g.C grids of g.g points.
+kp_status fft2_forward_pairs(const Fft2Plan* f, const Geom& g, kp_cdtype mt, const void* maps, const int2* pairs, float2* out,
+                             int64_t& launches, cudaStream_t st);
+Fft2Plan* fft2_make(int g0, int g1, int n1, kp_status* status);
+void fft2_free(Fft2Plan* f);
 // Inverse column pass of d_grid2 into the image rows of d_grid, clearing d_grid2; one of the two
 // row passes below completes the adjoint.
 kp_status fft2_inverse_cols(kp_plan p, cudaStream_t st);

@@ -67,3 +67,25 @@ def test_own_3d_fft_of_any_length(shape, C, kind):
     if C <= 3:
         assert rel(plan.make_preconditioner().cpu().numpy(), opc.mc_precond_fast(m, traj), "preconditioner") < 1e-5
     plan.close()
+
+
+# 2N grids 20x26 (13), 62x44 (31, 11), 34x96 (17), 48x36; one coil (a lone pair), coil counts that do and do not fill
+# the 4 coils of a thread, both line counts per CTA, every maps type
+@pytest.mark.parametrize("shape,C,kind", [((10, 13), 1, "c64"), ((31, 22), 3, "fp16"), ((17, 48), 4, "bf16"), ((24, 18), 9, "c64"),
+                                          ((64, 50), 13, "c64")])
+def test_preconditioner_pairs_and_coils(shape, C, kind):
+    """Pair products formed in the row pass, and the denominators of several coils at once."""
+    need_gpu()
+    import torch
+    from oracle import precond as opc
+    from paper_1902_09657_gb300.api import to_storage
+    M = 700
+    _, maps, traj = random_problem(shape, C, M, seed=C, edge=True)
+    md = to_storage(torch.from_numpy(maps).cuda(), kind)
+    plan = make_plan(shape, C, M)
+    plan.set_trajectory(to_dev(traj)).set_maps(md)
+    assert rel(plan.make_preconditioner(True).cpu().numpy(), opc.mc_precond_fast(rounded(md), traj), "mc") < 1e-5
+    sc = plan.make_preconditioner(False).cpu().numpy()
+    ref = opc.sc_precond_fast(traj, shape)
+    assert max(rel(sc[c], ref, "sc") for c in range(C)) < 1e-5
+    plan.close()
