@@ -357,12 +357,11 @@ def algorithmic_bytes(w, C, M, N, G, maps_bytes=8):
 # kernel code it was taken on; drop it when its kernel changes until it is captured again.
 NCU_TRAFFIC = {
     # one capture of the full 3D UTE workload (192^3 x 8 coils, 6,144,000 samples; one pass per
-    # kernel, so allowed at full size): KPDHG_SPREAD_VARIANT=10 KPDHG_SPREAD_CHUNK=256 ncu --metrics
-    # dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none
-    # -k "regex:k_spread_own|k_halo_gather" -s 10 -c 4 python bench.py --steps 1 --warmup 1 --no-extras
-    # k_spread_own<float2, 4>: 1.282 GB read + 1.440 GB written; k_halo_gather: 1.527 + 0.854 GB
-    ("ute3d_192", "spread"): {"bytes": 5103672448,
-                              "kernel": "k_spread_own<float2, 4> + k_halo_gather (one launch each, full 3D UTE workload)"},
+    # kernel, so allowed at full size): ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum
+    # --clock-control none -k regex:k_spread_cell3 -s 10 -c 2 python bench.py --steps 1 --warmup 1 --no-extras
+    ("ute3d_192", "spread"): {"bytes": 2521627648,
+                              "kernel": "k_spread_cell3<float2, 8> (one launch, full 3D UTE workload; 1.646 GB read, 0.876 GB "
+                                        "written; the clear of the grid before it, 0.885 GB, comes on top)"},
 }
 
 # Relative l2 errors against the float64 oracle measured by the GPU parity tests for the forms
@@ -580,8 +579,9 @@ def roofline(rc, ph):
     peak = float(peaks.get("hbm_gbs", 6800.0))
     achieved = ab[dom] / (own[dom] * 1e-3) / 1e9
     tr = NCU_TRAFFIC.get((w.name, dom))
-    kern = {"spread": "spreading (k_spread_own + k_halo_gather)" if "spread_reduce" in ph else "spreading",
-            "interp_dual": "k_interp_tile (interpolation + dual step)",
+    run = "spreading (k_spread_cell3)" if len(w.img_shape) == 3 else "spreading (k_spread_run)"
+    kern = {"spread": "spreading (k_spread_own + k_halo_gather)" if "spread_reduce" in ph else run,
+            "interp_dual": "interpolation + dual step (k_interp_run3 / k_interp_tile)",
             "adj_primal": "primal step (k_primal_fused / k_adj_primal)"}.get(dom, dom)
     out = {"kernel": kern, "phase": dom, "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
            "frac": achieved / peak, "traffic": tr["bytes"] if tr else None,

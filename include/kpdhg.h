@@ -100,7 +100,7 @@ const char* kp_status_string(kp_status s);
 const char* kp_last_error(void);
 
 /* Create a plan: validates `params`, allocates all device workspace (grids, sort buffers,
- * cuFFT plans) and uploads the apodisation and wavelet tables.  Synchronous.
+ * FFT plans) and uploads the apodisation and wavelet tables.  Synchronous.
  * Errors: KP_EINVAL (ndim not 2/3, non-positive sizes, width != 4, oversamp < 1,
  * levels incompatible with the image), KP_ENOMEM, KP_ECUFFT. */
 kp_status kp_plan_create(kp_plan* out, const kp_params* params, void* stream);
@@ -354,12 +354,12 @@ kp_status kp_batch_create(kp_batch* out, kp_plan* plans, int ncases);
  *   one case's FFTs overlap another case's interpolation or spreading.
  * KP_BATCH_PHASES: one kernel launch per phase over all cases (interpolation + dual step,
  *   split-tile clearing, spreading, primal step, each wavelet level, pre-step, counters; each
- *   block finds its case in a table of block offsets), with the cases' cuFFT transforms on
+ *   block finds its case in a table of block offsets), with the cases' transforms on
  *   forked streams between the phases.  Applies when every case is 2D, l2 or l1-wavelet, and
  *   the cases share one k-space and one maps storage type; otherwise the solve uses the
  *   per-case layout.  All cases spread with the single-pass interleaved-pair kernel.
- * On 64 uneven 2D cases (96..320 pixels, 4..32 coils) the per-case layout measured 7.1 ms per
- * iteration of all cases on a GB300 and the phase layout 8.7 ms. */
+ * The per-case layout is the faster one: its cases spread by runs and one case's kernels fill the
+ * gaps of another's. */
 typedef enum { KP_BATCH_PER_CASE = 0, KP_BATCH_PHASES = 1 } kp_batch_form;
 /* Selects the layout of later solves (the graph is captured again).  Errors: KP_EINVAL. */
 kp_status kp_batch_set_form(kp_batch batch, kp_batch_form form);

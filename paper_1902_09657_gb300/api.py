@@ -129,7 +129,7 @@ class Plan:
         return nt.value, mx.value
 
     def spread_config(self):
-        """Autotuned spreading choice: dict(variant, chunk, items, split_tiles)."""
+        """Spreading choice (by runs unless the environment asks for another): dict(variant, chunk, items, split_tiles)."""
         v, c, ni, ns = ctypes.c_int(), ctypes.c_int(), ctypes.c_int64(), ctypes.c_int64()
         L.check(self.lib.kp_plan_spread_config(self._h, ctypes.byref(v), ctypes.byref(c), ctypes.byref(ni),
                                                ctypes.byref(ns)), "kp_plan_spread_config")

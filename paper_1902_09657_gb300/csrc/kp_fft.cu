@@ -1,6 +1,8 @@
 // Own 3D FFT of a plan's oversampled grids (all coils at once), used in place of cuFFT for 3D
-// plans (any length with at most one prime factor above 5 and that up to 127) (Sec. 6's oversampled FFT, unnormalised in
-// both directions like cuFFT: forward e^{-2 pi i n k / g}, inverse e^{+2 pi i n k / g}).
+// plans whose lengths it factors (Sec. 6's oversampled FFT, unnormalised in both directions like cuFFT:
+// forward e^{-2 pi i n k / g}, inverse e^{+2 pi i n k / g}).  This file holds the passes compiled for one
+// length; an axis of another length (one prime factor above 5 at most, up to 127) takes the pass of
+// run-time length in kp_fft2.cu.
 //
 // One pass per axis.  A CTA takes 16 lines of one axis (8 for axes longer than 256 points): rows
 // along x, or columns along y or z for 16 (8) consecutive x, so every global access is a 128-
@@ -350,8 +352,8 @@ bool fftg_fits(const F2Axis& ax);
 template <int AXIS, bool INV, bool PRE, typename MT>
 kp_status fftg_pass(const F2Axis& ax, const FfConst& k, const Geom& g, const float2* in, float2* out, const PreSrc& pre, cudaStream_t st);
 
-// Passes and twiddle tables for grids of g[0] x g[1] x g[2] points; null when some length has no
-// compiled passes (or KPDHG_FFT=cufft).
+// Passes and twiddle tables for grids of g[0] x g[1] x g[2] points; null when some length has neither
+// compiled passes nor ones of run-time length (or KPDHG_FFT=cufft).
 Fft3Plan* fft3_make(const int g[3]) {
     const char* env = std::getenv("KPDHG_FFT");
     if (env && std::string(env) == "cufft") return nullptr;       // cuFFT when asked for
@@ -411,7 +413,7 @@ void fft3_destroy(kp_plan p) {
 
 // Grid sizes with compiled passes (the 3D workloads' grids and their preconditioner's 2N grids,
 // and small test grids); another length takes the passes of run-time length (150 x 132 x 116 x 5 coils,
-// grid 188 x 166 x 146 with the primes 47, 83 and 73: adjoint 1.33 ms, with cuFFT 1.79 ms).
+// grid 188 x 166 x 146 with the primes 47, 83 and 73: adjoint 1.38 ms, with cuFFT 1.79 ms).
 #define KP_FFT_SIZES(X) X(20) X(30) X(40) X(60) X(80) X(100) X(120) X(160) X(200) X(240) X(320) X(384) X(400) X(480)
 
 static bool size_compiled(int N) {

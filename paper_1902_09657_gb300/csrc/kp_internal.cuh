@@ -444,16 +444,17 @@ struct kp_plan_s {
     int* d_k0 = nullptr;             // [D][M] wrapped first tap ceil(t) - W/2 per sorted sample
     float* d_wt = nullptr;           // [D * W][M] Kaiser-Bessel weights per sorted sample
     int chunk = 256;                 // samples per interpolation work item (interp_items_chunk)
-    int spread_chunk = 256;          // samples per spreading work item (autotuned, multiple of 256)
+    int spread_chunk = 256;          // samples per spreading work item (per-tile variants; multiple of 256)
     int spread_variant = 0;          // 0/3/4/5: warp-private tiles (coils x warps 4x4, 2x8, 1x8, 2x4);
                                      // 1: shared atomics, 16 coils per CTA; 2: each warp owns 4 coils;
                                      // 6/7: warp-private interleaved coil pairs, 4 coils x 4 / 8 warps;
-                                     // 8/9: 3D z-plane owners; 10/11: 3D two-phase (padded tiles + gather)
+                                     // 8/9: 3D z-plane owners; 10/11: 3D two-phase (padded tiles + gather);
+                                     // 12: 2D two-phase; 13 (2D) / 14 (3D): runs, the default
     bool spread_tuned = false;
     int cluster_prox = -1;           // 2D l1 prox by one thread-block cluster: -1 unknown, 0 no, 1 yes
     int4* d_iitems = nullptr;        // interpolation work items {tile, begin, end, -1} over d_off ranges
     int64_t n_iitems = 0, iitems_cap = 0;
-    // two-phase 3D spreading (variants 10, 11): own-sample items, one padded-tile slot each
+    // own-sample items of the 3D run and the two-phase spreading (the latter: one padded-tile slot each)
     int4* d_oitems = nullptr;        // {tile, begin, end, slot} over d_off ranges, at most own_chunk samples
     int64_t n_oitems = 0, oitems_cap = 0;
     int* d_tslot = nullptr;          // [ntiles + 1] first slot of each tile

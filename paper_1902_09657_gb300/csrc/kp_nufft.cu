@@ -2,15 +2,16 @@
 // Sec. 6: Kaiser-Bessel gridding following Beatty et al., oversampling g/n, width 4).
 //
 // Forward:  pre-step (coil multiply, 1/Phi apodisation, centred zero padding) -> forward FFT
-//           of every coil's grid (2D: cuFFT; 3D: the own passes of kp_fft.cu, whose first pass
-//           forms the pre-step itself) -> interpolation (one CTA per (tile item, 4 coils), the
-//           tile's grid region staged in shared memory, one thread per sorted sample, W^D taps,
-//           N^{-1/2}).
-// Adjoint:  spreading into a second grid (variants chosen per plan by the autotuner: private
-//           tile copies per warp, or in 3D the two-phase padded tiles + gather; no zero-fill of
-//           the grid, split tiles cleared before they are accumulated) -> inverse FFT (cuFFT or
-//           the own passes, which leave only the crop valid) -> crop, 1/Phi, conj(s_c) coil
-//           combine, N^{-1/2} (fused into the primal step inside a PDHG iteration).
+//           of every coil's grid (the own passes of kp_fft2.cu in 2D and kp_fft.cu in 3D, whose
+//           first pass forms the pre-step itself; cuFFT for lengths they do not factor) ->
+//           interpolation (the tile's grid region staged in shared memory; 2D, and the last coils
+//           of 3D plans: one thread per sorted sample, W^D taps; 3D groups of 8 coils: runs of
+//           samples whose window values stay in registers; N^{-1/2}).
+// Adjoint:  spreading into a second grid (runs of sorted samples summed in registers over a
+//           moving window; the per-tile variants on request by the environment) -> inverse FFT
+//           (the own passes, which leave only the crop valid, or cuFFT) -> crop, 1/Phi, conj(s_c)
+//           coil combine, N^{-1/2} (fused into the last FFT pass in 2D and into the primal step
+//           inside a PDHG iteration).
 // The Kaiser-Bessel weights and first taps of every sample are tabulated once per
 // trajectory (sorted order, structure of arrays), so no Bessel function is evaluated
 // inside the iteration.
@@ -2828,13 +2829,14 @@ void spread_by_rule(kp_plan p) {
     p->spread_tuned = true;
 }
 
-// Picks the spreading variant and the samples per work item by timing the spreading kernels
-// on the plan's own work items (values do not affect the cost; once per plan, at its first
+// With a variant or an item size asked for by the environment: picks what was left open by timing the
+// spreading kernels on the plan's own work items (values do not affect the cost; once per plan, at its first
 // trajectory).  Variants: 0 private copies, 4 coils x 4 warps; 1 shared atomics; 2 warp per
 // 4 coils; 3 private, 2 coils x 8 warps; 4 private, 1 coil x 8 warps; 5 private, 2 coils x 4
 // warps; 6, 7 private interleaved coil pairs, 4 coils x 4 / 8 warps; 8, 9 (3D) z-plane owners,
 // 8 / 4 coils; 10, 11 (3D) two-phase padded tiles + gather, 8 / 4 coils, and 12 (2D) two-phase
-// with warp-private padded tiles (when their slot storage fits).  Larger items mean fewer split tiles (fewer global atomics) but fewer, longer CTAs.
+// with warp-private padded tiles (when their slot storage fits); 13 (2D) and 14 (3D) runs.  Larger items
+// mean fewer split tiles (fewer global atomics) but fewer, longer CTAs.
 kp_status autotune_spread(kp_plan p, cudaStream_t st) {
     if (p->spread_tuned) {
         // a new trajectory may need more slots than the two-phase variants hold: fall back to the

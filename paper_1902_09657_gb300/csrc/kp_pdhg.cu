@@ -5,7 +5,8 @@
 // inverse FFT -> fused primal kernel (adjoint combine, z = x - tau A^H u, l2 or l1-wavelet
 // prox, extrapolation, the next iteration's forward pre-step, iteration counter).  The step
 // sizes sigma_k, tau_k, theta_k are computed on the device in float64 from lambda_max and
-// min p, so one captured CUDA graph replays every iteration.
+// min p, so one captured CUDA graph replays every iteration in 3D.  2D plans on the own FFT
+// have the combine, primal step and pre-step inside its passes and issue their 4 to 7 kernels directly.
 #include "kp_internal.cuh"
 
 #include <cstdlib>

@@ -3,9 +3,9 @@
 // The trajectory step converts each sample to grid coordinates t_d = f_d * (g_d / n_d)
 // (float64, Sec. 6 NUFFT with oversampling g/n; kept as the first tap and a float32 offset),
 // sorts samples by the grid tile that
-// holds their first Kaiser-Bessel tap, and builds, per tile, the list of samples whose
-// W^D footprint touches that tile (used by the spreading kernel, which owns one output
-// tile per CTA and therefore needs no global atomics and no zero-fill of the grid).
+// holds their first Kaiser-Bessel tap and, inside a tile, by that tap's cell, which the run kernels
+// read as it is.  For the per-tile spreading variants (asked for by the environment, and the batch's
+// phase layout) it also builds, per tile, the list of samples whose W^D footprint touches that tile.
 #include "kp_internal.cuh"
 
 #include <algorithm>

@@ -1129,7 +1129,7 @@ static bool cluster_fits(size_t sm) {
 // Whether the 2D l1 prox can run as one cluster of 16 (else 8) CTAs: rows split evenly over
 // the CTAs with every level's row block even, shared memory within 200 KB, and the device able
 // to place the cluster.  The choice is made at solve set-up (outside any graph capture).  The
-// environment variable KPDHG_NO_CLUSTER_PROX=1 keeps the cooperative kernel.
+// environment variable KPDHG_NO_CLUSTER_PROX=1 keeps the level kernels (own 2D FFT) or the cooperative kernel.
 bool cluster_prox_ok(kp_plan p) {
     if (p->cluster_prox >= 0) return p->cluster_prox > 0;
     const Geom& g = p->geo;
